@@ -363,9 +363,10 @@ int dstd_conv_set_chunk_images(int max_images);
  * 8-byte records; 2 writes it out once per chunk, S [images, H, W, Mp, C_in]
  * in bf16 (the two nonzero grid weights of each input at grid steps k and
  * k + 1, zeros elsewhere), and the contractions read it through TMA boxes
- * shifted per filter tap; 0 (the default) writes S wherever its writer takes
- * the channel count (C_in <= 256, or a multiple of 256 up to 1024) and
- * generates elsewhere. Both compute the same products. It changes the workspace size, so query again after setting
+ * shifted per filter tap; 0 (the default) chooses per layer: forward and dS
+ * by source rows where that is faster (see dstd_conv_fwd), else S wherever
+ * its writer takes the channel count (C_in <= 256, or a multiple of 256 up to
+ * 1024) and generated elsewhere. All compute the same products. It changes the workspace size, so query again after setting
  * it. Returns the previous value (a policy outside 0..2 only reads it).
  * Process-wide; set it between calls. */
 int dstd_conv_set_operand_policy(int policy);

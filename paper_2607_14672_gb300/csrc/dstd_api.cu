@@ -736,11 +736,20 @@ int conv_fwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
                                        ws.rowsum, st)));
         }
     }
+    const bool cb_inner = !conv_fwd_row_boxes(gp, C_out, Mp);
+    const bool rows = g_conv_operand_policy == 0 && conv_rows_fwd_supported(gp, C_out, Mp, cb_inner);
     for (int img0 = 0; img0 < g.B; img0 += ws.imgs) {
         const int ni = (g.B - img0) < ws.imgs ? (g.B - img0) : ws.imgs;
         const long long in_off = (long long)img0 * g.H * g.W * g.C;
         const long long out_off = (long long)img0 * g.Ho * g.Wo * C_out;
         const long long P_out = (long long)ni * g.Ho * g.Wo;
+        if (rows) {  // binning, contraction and scan in one kernel
+            Timed tm(KK_GEMM_FWD, st);
+            TRY(cu(launch_conv_rows_fwd(gp, ni, C_out, c, cb_inner, t_in + in_off, g.C, ws.Wf, ws.rowsum,
+                                        t_out + out_off, sv.q + out_off, sv.s + out_off, sv.vdot + out_off, penalty,
+                                        st)));
+            continue;
+        }
         {
             Timed tm(KK_BIN, st);
             if (ws.S)
@@ -796,7 +805,10 @@ int conv_bwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
         }
         if (g_t_in) {
             Timed tm(KK_GEMM_DS, st);
-            TRY(cu(launch_conv_ds_gemm(gp, ni, C_out, c, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off, g.C, st)));
+            if (g_conv_operand_policy == 0 && conv_rows_ds_supported(gp, C_out, Mp))
+                TRY(cu(launch_conv_rows_ds(gp, ni, C_out, c, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off, g.C, st)));
+            else
+                TRY(cu(launch_conv_ds_gemm(gp, ni, C_out, c, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off, g.C, st)));
         }
         {
             Timed tm(KK_BIN_T, st);
@@ -1637,6 +1649,9 @@ int dstd_device_status(int clear) {
     unsigned int s = 0, s2 = 0;
     if (status_read(&s, clear) != cudaSuccess) return DSTD_E_CUDA;
     if (conv_status_read(&s2, clear) != cudaSuccess) return DSTD_E_CUDA;
+    unsigned int s3 = 0;
+    if (conv_rows_status_read(&s3, clear) != cudaSuccess) return DSTD_E_CUDA;
+    s2 |= s3;
     return ((s | s2) & STATUS_TIMEOUT) ? DSTD_E_TIMEOUT : DSTD_OK;
 }
 

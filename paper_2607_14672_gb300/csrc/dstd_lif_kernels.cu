@@ -49,6 +49,7 @@ LifConst make_const(const dstd_params &p, int Mp) {
         const double s4 = tp < 4.0 * dt ? tp : 4.0 * dt;
         const double phi4 = lam == 0.0 ? s4 : -expm1(-lam * s4) / lam;
         c.Kmax4 = (float)(exp(-av * s4) * phi4 * (1.0 + 1e-6));
+        c.fall = (float)(exp(av * dt) * (1.0 + 1e-5));
     }
     c.t_head = p.t_head;
     c.t_tail = p.t_tail;

@@ -171,6 +171,106 @@ static __device__ __forceinline__ void mma_commit(uint64_t *bar) {
                  : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// Issue by a whole warp. tcgen05.mma, its commit and TMA copies take their
+// descriptors, addresses and coordinates from uniform registers. In a branch
+// that one lane takes, with an exit that depends on a wait's result, the
+// compiler cannot tell that they are uniform: an MMA then costs 102 clocks to
+// issue whatever its size (measured: M = 128, N = 64, 4 MMAs per wait; the
+// tensor core itself takes 48, and 64 with N = 128). So every lane runs the
+// loop, waits end it by a warp vote, and only the instructions are left to the
+// elected lane (68 clocks with 4 MMAs per wait, 54 with 36).
+// ---------------------------------------------------------------------------
+static __device__ __forceinline__ uint32_t elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(p));
+    return p;
+}
+
+// a value that is the same in every lane, through a warp reduction, whose
+// result the compiler knows to be uniform
+static __device__ __forceinline__ uint32_t uniform(uint32_t x) { return __reduce_or_sync(0xffffffffu, x); }
+
+// bounded wait of a whole warp: the same answer in every lane
+static __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity) {
+    return !__any_sync(0xffffffffu, !mbar_wait_spin(bar, parity));
+}
+
+// An MMA (inside a branch of the elected lane) with descriptors given by their
+// low words (start address / 16, and the encoded leading offset): the high word of a K-major 128-byte-swizzle
+// descriptor is a constant, so stepping an operand is one addition
+constexpr uint32_t SDESC_KK_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
+static __device__ __forceinline__ uint32_t sdesc_kk_lo(uint32_t saddr) {
+    return ((saddr & 0x3FFFFu) >> 4) | (1u << 16);
+}
+static __device__ __forceinline__ void mma_kk(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                              uint32_t accumulate) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        ".reg .b64 da, db;\n"
+        "mov.b64 da, {%1, %3};\n"
+        "mov.b64 db, {%2, %3};\n"
+        "setp.ne.b32 p, %5, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n"
+        "}\n" ::"r"(d_tmem),
+        "r"(alo), "r"(blo), "r"(SDESC_KK_HI), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+static __device__ __forceinline__ void mma_commit_if(uint32_t lead, uint64_t *bar) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(smem_u32(bar)),
+        "r"(lead)
+        : "memory");
+}
+
+static __device__ __forceinline__ void mbar_expect_tx_if(uint32_t lead, uint64_t *bar, uint32_t bytes) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %2, 0;\n"
+        "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+        "}\n" ::"r"(smem_u32(bar)),
+        "r"(bytes), "r"(lead)
+        : "memory");
+}
+
+static __device__ __forceinline__ void tma_load_2d_if(uint32_t lead, uint32_t dst, const CUtensorMap *map, uint64_t *bar,
+                                                      int x, int y) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %5, 0;\n"
+        "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
+        "}\n" ::"r"(dst),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar)), "r"(lead)
+        : "memory");
+}
+
+static __device__ __forceinline__ void tma_load_5d_if(uint32_t lead, uint32_t dst, const CUtensorMap *map, uint64_t *bar,
+                                                      int c, int m, int x, int y, int b) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %8, 0;\n"
+        "@q cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n"
+        "}\n" ::"r"(dst),
+        "l"((uint64_t)map), "r"(c), "r"(m), "r"(x), "r"(y), "r"(b), "r"(smem_u32(bar)), "r"(lead)
+        : "memory");
+}
+
 // 32 lanes x 32 consecutive fp32 columns; the wait is in the same asm block
 // so the registers are valid when the statement completes.
 static __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
