@@ -737,15 +737,20 @@ int conv_fwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
         }
     }
     const bool cb_inner = !conv_fwd_row_boxes(gp, C_out, Mp);
-    const bool rows = g_conv_operand_policy == 0 && conv_rows_fwd_supported(gp, C_out, Mp, cb_inner);
+    const bool rows = g_conv_operand_policy == 0 && ws.S && conv_rows_fwd_supported(gp, C_out, Mp, cb_inner);
     for (int img0 = 0; img0 < g.B; img0 += ws.imgs) {
         const int ni = (g.B - img0) < ws.imgs ? (g.B - img0) : ws.imgs;
         const long long in_off = (long long)img0 * g.H * g.W * g.C;
         const long long out_off = (long long)img0 * g.Ho * g.Wo * C_out;
         const long long P_out = (long long)ni * g.Ho * g.Wo;
-        if (rows) {  // binning, contraction and scan in one kernel
+        if (rows) {  // 8 bytes per input (in S's place, which is larger), then contraction and scan in one kernel
+            uint2 *rec = reinterpret_cast<uint2 *>(ws.S);
+            {
+                Timed tm(KK_BIN, st);
+                TRY(cu(launch_bin_rec(t_in + in_off, (long long)ni * g.H * g.W * g.C, c, rec, st)));
+            }
             Timed tm(KK_GEMM_FWD, st);
-            TRY(cu(launch_conv_rows_fwd(gp, ni, C_out, c, cb_inner, t_in + in_off, g.C, ws.Wf, ws.rowsum,
+            TRY(cu(launch_conv_rows_fwd(gp, ni, C_out, c, cb_inner, rec, g.C, ws.Wf, ws.rowsum,
                                         t_out + out_off, sv.q + out_off, sv.s + out_off, sv.vdot + out_off, penalty,
                                         st)));
             continue;

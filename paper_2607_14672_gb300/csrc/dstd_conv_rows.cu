@@ -12,14 +12,13 @@
 // box serves 36 to 72 MMAs. What bounds this kernel then: dS at 64 channels
 // runs at 53 clocks per N = 64 MMA, of which reading the operands from shared
 // memory takes 48 (64 -> 64 at 28 x 28, B = 256, M = 64: 1.35 -> 0.68 ms); the
-// forward is bound by the instructions of the generators and the scan, which
-// keep the SM's issue slots 60 to 76% busy (the same layer: 2.38 -> 1.82 ms
+// forward is bound by the scan's instructions (the same layer: 2.38 -> 1.75 ms
 // with the binning).
 //
-//   forward  the box holds the binned input and is generated on chip from the
-//            spike times (two nonzeros of Mp per input; generator warps erase
+//   forward  the box holds the binned input and is generated on chip from 8
+//            bytes per input spike (two nonzeros of Mp; generator warps erase
 //            the last ones and write the new), so no binned input is written
-//            to memory at all; the epilogue runs the scan/solve/select;
+//            to memory; the epilogue runs the scan/solve/select;
 //   dS       the box holds dw^ rows, loaded by TMA; the epilogue takes the
 //            input-time gradient.
 //
@@ -59,7 +58,7 @@ constexpr int MMA_WARPS = 4;   // issuing warps: output row n by warp n mod 4
 constexpr int GEN_SLOTS = 7;   // (position, channel) slots of a generator thread per box, at most
 constexpr int EPI_LDF = 36;    // forward epilogue: floats per neuron row of 32 grid steps (read as float4)
 constexpr int EPI_LDG = 33;    // dS epilogue: floats per grid-step row of 32 channels
-constexpr int SILENT = -128;   // kept grid step of a slot that holds no spike
+constexpr int SILENT = -128;   // grid step of a record, and kept step of a slot, without a spike
 
 struct RowsPlan {
     int n_items, n_xt, n_col, n_strip, R;  // items; position tiles, column tiles, strips of R output rows
@@ -77,7 +76,8 @@ struct RowsPlan {
 };
 
 struct RowsArgs {
-    const float *t_in;  // source spike times (forward), or the layer input's (dS): C_t channels
+    const uint2 *rec;   // forward: the source's records (k_bin_rec), C_t channels
+    const float *t_in;  // dS: the layer input's spike times, C_t channels
     int C_t;
     int C_out;          // channels of the output grid (forward: C_out; dS: C_in padded)
     float *t_out;       // forward
@@ -91,11 +91,6 @@ struct RowsArgs {
 
 __host__ __device__ constexpr uint32_t idesc_kk(int N) {  // M = 128, both operands K-major bf16
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-}
-
-__device__ __forceinline__ uint32_t rows_pack_bf16x2(float a, float b) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t *>(&h);
 }
 
 __device__ __forceinline__ void rows_sts_u16(uint32_t addr, uint16_t v) {
@@ -425,7 +420,10 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
 
     if (FWD && warp < GEN_WARPS) {
         // Generators: thread (g, c) writes channel c of the box positions
-        // g, g + 2, ...; its spike times are loaded one box ahead.
+        // g, g + 2, ...; its records are loaded one box ahead. (The weights are
+        // computed once per input by k_bin_rec: computed here, twice or more
+        // per input, they took a quarter of the kernel's issue slots and left
+        // the generators 3600 clocks per box.)
         const int g0 = threadIdx.x >> 6, c = threadIdx.x & 63;
         Item<FWD> nx;
         int n_it = blockIdx.x, n_sr = 0, n_cb = 0;
@@ -433,16 +431,16 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
             nx.decode(p, n_it);
             n_sr = nx.sr;
         }
-        float tn[SLOTS];
+        uint2 tn[SLOTS];
         auto load_next = [&]() {
             const int ch = n_cb * 64 + c;
             const bool on = n_it < p.n_items && ch < a.C_t;
             const int x0 = on ? nx.xt * p.xs_mul + p.xs_add : 0;
-            const float *src = on ? a.t_in + (((long long)nx.b * p.sh + n_sr) * p.sw + x0) * a.C_t + ch : nullptr;
+            const uint2 *src = on ? a.rec + (((long long)nx.b * p.sh + n_sr) * p.sw + x0) * a.C_t + ch : nullptr;
 #pragma unroll
             for (int u = 0; u < SLOTS; ++u) {
                 const int i = g0 + 2 * u;
-                tn[u] = INFINITY;
+                tn[u] = make_uint2((uint32_t)SILENT, 0u);
                 if (on && i < p.npos && x0 + i >= 0 && x0 + i < p.sw) tn[u] = __ldg(src + (long long)i * a.C_t);
             }
             if (n_it < p.n_items && ++n_cb == ncb) {
@@ -467,9 +465,9 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
             for (int sr = w.sr; !w.done(sr) && ok; ++sr) {
                 for (int cbo = 0; cbo < cbo_n; ++cbo) {
                     for (int cbi = 0; cbi < cbi_n; ++cbi) {
-                        float tc_[SLOTS];
+                        uint2 cur[SLOTS];
 #pragma unroll
-                        for (int u = 0; u < SLOTS; ++u) tc_[u] = tn[u];
+                        for (int u = 0; u < SLOTS; ++u) cur[u] = tn[u];
                         load_next();
                         if (cbi == 0) {  // the stage's previous MMAs are done with it
                             int got = 1;
@@ -482,23 +480,12 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                         }
                         const uint32_t box = tc::smem_u32(smem + sa * p.stage_bytes + cbi * p.box_bytes);
                         int8_t *kp = kept + ((sa * cbi_n + cbi) * p.npos) * 64 + c;
-                        // not unrolled: one copy of the weights' code
-#pragma unroll 1
+#pragma unroll
                         for (int u = 0; u < SLOTS; ++u) {
                             const int i = g0 + 2 * u;
                             if (i >= p.npos) break;
-                            float t = tc_[0];
-#pragma unroll
-                            for (int z = 1; z < SLOTS; ++z) t = u == z ? tc_[z] : t;
-                            int kk = SILENT;
-                            uint32_t wq = 0u;
-                            if (isfinite(t)) {
-                                const BinW bw = bin_weights(a.c, t, false);
-                                if (bw.k >= -1 && bw.k < a.c.M) {
-                                    kk = bw.k;
-                                    wq = rows_pack_bf16x2(bw.wR, bw.wL);
-                                }
-                            }
+                            const int kk = (int)cur[u].x;
+                            const uint32_t wq = cur[u].y;
                             const int place = planes == 1 ? i : (i & 1) * per_plane + (i >> 1);
                             const int row0 = place * Mp, old = kp[i * 64];
                             if (old != SILENT) {
@@ -1213,13 +1200,13 @@ bool conv_rows_fwd_supported(const ConvGeom &g, int C_out, int Mp, bool cb_inner
 }
 
 cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
-                                 const float *t_in, int C_t, const __nv_bfloat16 *Wf, const float *rowsum,
+                                 const uint2 *rec, int C_t, const __nv_bfloat16 *Wf, const float *rowsum,
                                  float *t_out, int *q, float *s, float *vdot, float *penalty, cudaStream_t st) {
     RowsPlan p;
     Tile t;
     if (!rows_pick(true, g, ni, C_out, c.Mp, cb_inner, p, t)) return cudaErrorInvalidConfiguration;
     RowsArgs a{};
-    a.t_in = t_in;
+    a.rec = rec;
     a.C_t = C_t;
     a.C_out = C_out;
     a.t_out = t_out;

@@ -504,11 +504,11 @@ cudaError_t launch_conv_fwd_tma(const ConvGeom &g, int ni, int C_out, const LifC
 bool conv_fwd_row_boxes(const ConvGeom &g, int C_out, int Mp);
 // The forward and dS contractions that take each source row once
 // (dstd_conv_rows.cu): same results (the forward generates the binned input on
-// chip from t_in [ni H W][C_t]; cb_inner as conv_fwd_row_boxes says, so that
+// chip from the records of launch_bin_rec, [ni H W][C_t]; cb_inner as conv_fwd_row_boxes says, so that
 // w^ is the same bit for bit). supported: the shapes they take.
 bool conv_rows_fwd_supported(const ConvGeom &g, int C_out, int Mp, bool cb_inner);
 cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
-                                 const float *t_in, int C_t, const __nv_bfloat16 *Wf, const float *rowsum,
+                                 const uint2 *rec, int C_t, const __nv_bfloat16 *Wf, const float *rowsum,
                                  float *t_out, int *q, float *s, float *vdot, float *penalty, cudaStream_t st);
 bool conv_rows_ds_supported(const ConvGeom &g, int C_out, int Mp);
 cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *dW_hat,
