@@ -897,6 +897,19 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_3d_if(uint32_t lead, uint32_t dst, const CUtensorMap *map, uint64_t *bar, int c,
+                                               int m, int p) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %6, 0;\n"
+        "@q cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];\n"
+        "}\n" ::"r"(dst),
+        "l"((uint64_t)map), "r"(c), "r"(m), "r"(p), "r"(tc::smem_u32(bar)), "r"(lead)
+        : "memory");
+}
+
 __device__ __forceinline__ void sts_u16(uint32_t addr, uint16_t v) {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
 }
@@ -1598,9 +1611,18 @@ __global__ void __launch_bounds__(DW_THREADS, 1)
 // 2-9 epilogue (fp32 atomics into g_W, dead-neuron term on the first split).
 // ---------------------------------------------------------------------------
 constexpr int DWT_MAX_STAGES = 8;
+// The row tiles of a K step go round the issuing warps (each tile its own
+// accumulator, always the same warp): between the MMAs of two K steps a warp
+// spends some 500 clocks on waits and addresses, which the others cover. With
+// one warp, whose operands the compiler could not keep in uniform registers, an
+// N = 64 MMA took 90 clocks over the whole loop (64 -> 64 at 28 x 28, B = 256,
+// M = 64: 1.49 -> 1.29 ms; 512 -> 512 at 4 x 4, B = 128, M = 32: 307 -> 236
+// us; what bounds them now is loading a box per tap, two stages in flight).
+constexpr int DWT_MMA_WARPS = 4;
+constexpr int DWT_THREADS = (1 + DWT_MMA_WARPS + CONV_NEPI) * 32;
 
 template <int BN>
-__global__ void __launch_bounds__(CONV_THREADS, 1)
+__global__ void __launch_bounds__(DWT_THREADS, 1)
     k_conv_dw_tma(const __grid_constant__ CUtensorMap mapS, const __grid_constant__ CUtensorMap mapD, ConvGemmArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1627,9 +1649,9 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     if (threadIdx.x == 0) {
         for (int s = 0; s < NST; ++s) {
             tc::mbar_init(&full[s], 1);
-            tc::mbar_init(&empty[s], 1);
+            tc::mbar_init(&empty[s], DWT_MMA_WARPS);
         }
-        tc::mbar_init(acc_full, 1);
+        tc::mbar_init(acc_full, DWT_MMA_WARPS);
         tc::mbar_init(acc_empty, CONV_NEPI);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1650,7 +1672,8 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     };
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
+            const uint32_t lead = tc::elect_one();
             const uint32_t tx = (uint32_t)(STG);  // 2G row blocks x kpos boxes of Mp x 128 B, and the dw^ tile
             uint32_t it = 0;
             int s = 0;
@@ -1677,12 +1700,11 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                 int p = kt0 * kpos, b, y, x;
                 pos_decode(p, a.Ho, a.Wo, b, y, x);
                 for (int i = 0; i < nkt; ++i, ++it) {
-                    if (!tc::mbar_wait_spin(&empty[s], ph ^ 1u)) {
-                        conv_set_status(STATUS_TIMEOUT);
+                    if (!tc::mbar_wait_warp(&empty[s], ph ^ 1u)) {
                         ok = false;
                         break;
                     }
-                    tc::mbar_expect_tx(&full[s], tx);
+                    tc::mbar_expect_tx_if(lead, &full[s], tx);
                     const uint32_t st = tc::smem_u32(smem + s * STG);
                     for (int kp = 0; kp < kpos; ++kp) {
                         const bool pv = p < a.P_rows;
@@ -1693,7 +1715,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                                 // a row block past the filter rows or a position past the
                                 // chunk reads a box outside the tensor (zeros)
                                 const bool on = pv && rkh[u] >= 0;
-                                tma_load_5d(st + (u >> 1) * 16384 + (u & 1) * 8192 + kp * Mp * 128, &mapS, &full[s],
+                                tc::tma_load_5d_if(lead, st + (u >> 1) * 16384 + (u & 1) * 8192 + kp * Mp * 128, &mapS, &full[s],
                                             rcb[u] * 64, 0, on ? xs + rkw[u] : 0, on ? ys + rkh[u] : 0, on ? b : a.ni);
                             }
                         }
@@ -1708,64 +1730,71 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                     }
                     const uint32_t sb = st + a_bytes;
                     for (int gq = 0; gq < BN / 64; ++gq)
-                        tma_load_3d(sb + gq * 8192, &mapD, &full[s], ct * BN + gq * 64, 0, (kt0 + i) * kpos);
+                        tma_load_3d_if(lead, sb + gq * 8192, &mapD, &full[s], ct * BN + gq * 64, 0, (kt0 + i) * kpos);
                     if (++s == NST) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
             }
+            if (!ok && lead) conv_set_status(STATUS_TIMEOUT);
             const uint32_t n_drain = it < (uint32_t)NST ? it : (uint32_t)NST;
             for (uint32_t i = it - n_drain; i < it; ++i) tc::mbar_wait_spin(&full[i % NST], (i / NST) & 1u);
         }
         __syncwarp();
-    } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(128, BN, true, true);
-            uint32_t j = 0;
-            int s = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++j) {
-                int rg, ct, kt0, nkt;
-                decode(t, rg, ct, kt0, nkt);
-                if (j >= 1) {
-                    if (!tc::mbar_wait_spin(acc_empty, (j - 1) & 1u)) {
-                        conv_set_status(STATUS_TIMEOUT);
-                        break;
-                    }
-                    tc::tc_fence_after();
+    } else if (warp <= DWT_MMA_WARPS) {
+        const int mw = warp - 1;
+        const uint32_t lead = tc::elect_one();
+        constexpr uint32_t idesc = idesc_bf16(128, BN, true, true);
+        // low descriptor words (start address / 16, the 8 KB to the next 64
+        // columns) stepped by additions: a row tile is 16 KB on, a 16-deep slice 2 KB
+        constexpr uint32_t HI = (uint32_t)(tc::sdesc_sw128_mn_hi());
+        const uint32_t base = ((tc::smem_u32(smem) & 0x3FFFFu) >> 4) | ((8192u >> 4) << 16);
+        const uint32_t tmem_u = tc::uniform(tmem);
+        uint32_t j = 0;
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++j) {
+            int rg, ct, kt0, nkt;
+            decode(t, rg, ct, kt0, nkt);
+            if (j >= 1) {
+                if (!tc::mbar_wait_warp(acc_empty, (j - 1) & 1u)) {
+                    ok = false;
+                    break;
                 }
-                for (int i = 0; i < nkt; ++i) {
-                    if (!tc::mbar_wait_spin(&full[s], ph)) {
-                        conv_set_status(STATUS_TIMEOUT);
-                        ok = false;
-                        break;
-                    }
-                    tc::tc_fence_after();
-                    const uint32_t sa = tc::smem_u32(smem + s * STG);
-                    const uint32_t sbb = sa + a_bytes;
-                    // descriptors built once: a row tile is 16 KB on (+1024), a
-                    // 16-deep slice 2 KB (+128)
-                    const uint64_t ad0 = tc::sdesc_sw128_mn(sa, 8192), bd0 = tc::sdesc_sw128_mn(sbb, 8192);
-                    for (int gi = 0; gi < G; ++gi) {
+                tc::tc_fence_after();
+            }
+            for (int i = 0; i < nkt; ++i) {
+                if (!tc::mbar_wait_warp(&full[s], ph)) {
+                    ok = false;
+                    break;
+                }
+                tc::tc_fence_after();
+                const uint32_t alo = tc::uniform(base + (uint32_t)(s * (STG >> 4)));
+                const uint32_t blo = alo + (uint32_t)(a_bytes >> 4);
+                const uint32_t more = i > 0 ? 1u : 0u;
+                if (lead) {
+                    for (int gi = mw; gi < G; gi += DWT_MMA_WARPS) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
-                            tc::mma_bf16(tmem + gi * BN, ad0 + (uint64_t)(gi * 1024 + kk * 128), bd0 + (uint64_t)(kk * 128),
-                                         idesc, (i > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    tc::mma_commit(&empty[s]);
-                    if (++s == NST) {
-                        s = 0;
-                        ph ^= 1u;
+                            tc::mma_lo<HI>(tmem_u + gi * BN, alo + (uint32_t)(gi * 1024 + kk * 128),
+                                           blo + (uint32_t)(kk * 128), idesc, kk > 0 ? 1u : more);
                     }
                 }
-                if (ok) tc::mma_commit(acc_full);
+                __syncwarp();
+                tc::mma_commit_if(lead, &empty[s]);
+                if (++s == NST) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
+            if (ok) tc::mma_commit_if(lead, acc_full);
         }
+        if (!ok && lead) conv_set_status(STATUS_TIMEOUT);
         __syncwarp();
     } else {
-        const int quarter = warp & 3, group = (warp - 2) >> 2;
+        const int quarter = warp & 3, group = (warp - 1 - DWT_MMA_WARPS) >> 2;
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         const int r = quarter * 32 + lane;
         uint32_t j = 0;
@@ -2210,7 +2239,7 @@ cudaError_t launch_conv_dw_tma(const ConvGeom &g, int ni, int C_out, const LifCo
     {                                                                                                            \
         cudaError_t e = cudaFuncSetAttribute(k_conv_dw_tma<BNV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); \
         if (e != cudaSuccess) return e;                                                                          \
-        k_conv_dw_tma<BNV><<<grid, CONV_THREADS, smem, st>>>(mS, mD, a);                                         \
+        k_conv_dw_tma<BNV><<<grid, DWT_THREADS, smem, st>>>(mS, mD, a);                                         \
         return cudaGetLastError();                                                                               \
     }
     switch (BN) {

@@ -209,7 +209,10 @@ constexpr uint32_t SDESC_KK_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 static __device__ __forceinline__ uint32_t sdesc_kk_lo(uint32_t saddr) {
     return ((saddr & 0x3FFFFu) >> 4) | (1u << 16);
 }
-static __device__ __forceinline__ void mma_kk(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
+// (the MN-major 128-byte-swizzle descriptor has the same high word)
+static __host__ __device__ constexpr uint32_t sdesc_sw128_mn_hi() { return SDESC_KK_HI; }
+template <uint32_t HI>
+static __device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
                                               uint32_t accumulate) {
     asm volatile(
         "{\n"
@@ -220,8 +223,12 @@ static __device__ __forceinline__ void mma_kk(uint32_t d_tmem, uint32_t alo, uin
         "setp.ne.b32 p, %5, 0;\n"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n"
         "}\n" ::"r"(d_tmem),
-        "r"(alo), "r"(blo), "r"(SDESC_KK_HI), "r"(idesc), "r"(accumulate)
+        "r"(alo), "r"(blo), "r"(HI), "r"(idesc), "r"(accumulate)
         : "memory");
+}
+static __device__ __forceinline__ void mma_kk(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                              uint32_t accumulate) {
+    mma_lo<SDESC_KK_HI>(d_tmem, alo, blo, idesc, accumulate);
 }
 
 static __device__ __forceinline__ void mma_commit_if(uint32_t lead, uint64_t *bar) {
