@@ -737,13 +737,13 @@ int conv_fwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
         }
     }
     const bool cb_inner = !conv_fwd_row_boxes(gp, C_out, Mp);
-    const bool rows = g_conv_operand_policy == 0 && ws.S && conv_rows_fwd_supported(gp, C_out, Mp, cb_inner);
     for (int img0 = 0; img0 < g.B; img0 += ws.imgs) {
         const int ni = (g.B - img0) < ws.imgs ? (g.B - img0) : ws.imgs;
         const long long in_off = (long long)img0 * g.H * g.W * g.C;
         const long long out_off = (long long)img0 * g.Ho * g.Wo * C_out;
         const long long P_out = (long long)ni * g.Ho * g.Wo;
-        if (rows) {  // 8 bytes per input (in S's place, which is larger), then contraction and scan in one kernel
+        if (g_conv_operand_policy == 0 && ws.S && conv_rows_fwd_supported(gp, ni, C_out, Mp, cb_inner)) {
+            // 8 bytes per input (in S's place, which is larger), then contraction and scan in one kernel
             uint2 *rec = reinterpret_cast<uint2 *>(ws.S);
             {
                 Timed tm(KK_BIN, st);
@@ -810,8 +810,10 @@ int conv_bwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
         }
         if (g_t_in) {
             Timed tm(KK_GEMM_DS, st);
-            if (g_conv_operand_policy == 0 && conv_rows_ds_supported(gp, C_out, Mp))
-                TRY(cu(launch_conv_rows_ds(gp, ni, C_out, c, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off, g.C, st)));
+            const bool cb_inner = !conv_ds_row_boxes(gp, C_out, Mp);
+            if (g_conv_operand_policy == 0 && conv_rows_ds_supported(gp, ni, C_out, Mp, cb_inner))
+                TRY(cu(launch_conv_rows_ds(gp, ni, C_out, c, cb_inner, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off,
+                                           g.C, st)));
             else
                 TRY(cu(launch_conv_ds_gemm(gp, ni, C_out, c, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off, g.C, st)));
         }

@@ -1162,24 +1162,25 @@ struct Tile {
 };
 
 // The tile shapes to try, best first, where this kernel is the faster one.
-// Measured against the one-row-at-a-time kernels, every layer shape of the
-// 9- and 20-layer networks at their batches:
-//   forward  64 output channels: 1.02 to 1.28 times faster (binning included);
-//            128 and more, whose filters stream through shared memory: 0.69 to
-//            1.06, so they stay there;
-//   dS       64 input channels: 1.1 to 2.6 times faster (64 -> 64 at 28 x 28:
-//            1.86; 64 -> 128 at stride 2: 2.5); 128 input channels: 1.0 to 1.24
-//            with up to 128 output channels, 0.8 to 0.9 with 256; wider: 0.5 to
-//            0.9 (the filters of a column tile are read once per source row).
+// Measured against the one-row-at-a-time kernels (whose issue loops run as
+// whole warps too), every layer shape of the 9- and 20-layer networks:
+//   forward  64 output channels of one channel block at stride 1: 1.01 to 1.07
+//            times faster from about 300 output positions per SM on (binning
+//            included), 0.86 to 0.96 below; two channel blocks 0.82, stride 2
+//            0.95 to 1.02, 1x1 0.91, 128 and more output channels (filters
+//            streamed): 0.6 to 0.9;
+//   dS       64 input channels: 1.2 to 2.3 times faster (64 -> 64 at 28 x 28:
+//            1.55; 64 -> 128 at stride 2: 2.0), 0.87 to 1 on a few thousand
+//            positions; 128 input channels: 0.8 to 0.96, wider: 0.5 to 0.9.
 bool rows_pick(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner, RowsPlan &p, Tile &t) {
     Tile tr[3];
     int n = 0;
     if (fwd) {
-        if (C_out != 64) return false;
+        if (C_out != 64 || g.C != 64 || g.s != 1 || g.k == 1) return false;
+        if ((long long)ni * g.Ho * g.Wo < 300ll * rows_num_sms()) return false;
         for (int nset = 4; nset >= 2; --nset) tr[n++] = {64, 1, nset};
     } else {
-        if (g.C > 128 || (g.C == 128 && C_out > 128)) return false;
-        if (g.s == 1 && g.C == 128) tr[n++] = {128, 1, 2};
+        if (g.C != 64 || (long long)ni * g.H * g.W < 20ll * rows_num_sms()) return false;
         tr[n++] = {64, 2, 2};
         tr[n++] = {64, 1, 2};
     }
@@ -1193,10 +1194,10 @@ bool rows_pick(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_i
 
 }  // namespace
 
-bool conv_rows_fwd_supported(const ConvGeom &g, int C_out, int Mp, bool cb_inner) {
+bool conv_rows_fwd_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner) {
     RowsPlan p;
     Tile t;
-    return rows_pick(true, g, 1, C_out, Mp, cb_inner, p, t);
+    return rows_pick(true, g, ni, C_out, Mp, cb_inner, p, t);
 }
 
 cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
@@ -1221,17 +1222,17 @@ cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const Lif
     return rows_launch<64, 1, true>(mB, mB, a, p, st);
 }
 
-bool conv_rows_ds_supported(const ConvGeom &g, int C_out, int Mp) {
+bool conv_rows_ds_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner) {
     RowsPlan p;
     Tile t;
-    return rows_pick(false, g, 1, C_out, Mp, false, p, t);
+    return rows_pick(false, g, ni, C_out, Mp, cb_inner, p, t);
 }
 
-cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *dW_hat,
-                                const __nv_bfloat16 *Wt, const float *t_in, float *g_t_in, int C_t, cudaStream_t st) {
+cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
+                                const __nv_bfloat16 *dW_hat, const __nv_bfloat16 *Wt, const float *t_in, float *g_t_in, int C_t, cudaStream_t st) {
     RowsPlan p;
     Tile t;
-    if (!rows_pick(false, g, ni, C_out, c.Mp, false, p, t)) return cudaErrorInvalidConfiguration;
+    if (!rows_pick(false, g, ni, C_out, c.Mp, cb_inner, p, t)) return cudaErrorInvalidConfiguration;
     cudaError_t e = cudaMemsetAsync(g_t_in, 0, sizeof(float) * (size_t)ni * g.H * g.W * C_t, st);
     if (e != cudaSuccess) return e;
     RowsArgs a{};
@@ -1244,7 +1245,6 @@ cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifC
     if (!rows_map_act(&mA, dW_hat, ni, g.Ho, g.Wo, c.Mp, C_out, p.npos) ||
         !rows_map_mat(&mB, Wt, g.C, g.k * g.k * C_out, t.BN))
         return cudaErrorInvalidValue;
-    if (t.BN == 128) return rows_launch<128, 1, false>(mA, mB, a, p, st);
     if (t.NT == 2) return rows_launch<64, 2, false>(mA, mB, a, p, st);
     return rows_launch<64, 1, false>(mA, mB, a, p, st);
 }

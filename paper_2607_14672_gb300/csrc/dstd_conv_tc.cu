@@ -272,18 +272,6 @@ __global__ void k_filters_t(const float *__restrict__ W, int C_out, int T, int C
 }
 
 
-// ---------------------------------------------------------------------------
-// TMA loads of 5-D boxes (channel, m, x, y, b) into this CTA's shared memory
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, uint64_t *bar, int c, int m, int x,
-                                            int y, int b) {
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
-        "l"((uint64_t)map), "r"(c), "r"(m), "r"(x), "r"(y), "r"(b), "r"(tc::smem_u32(bar))
-        : "memory");
-}
-
 // Instruction descriptor, kind::f16 with bf16 A and B and fp32 D; a_mn / b_mn
 // select MN-major operands (transpose bits 15 and 16).
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn, bool b_mn) {
@@ -396,15 +384,19 @@ __host__ __device__ constexpr int fwd_epi_bytes(bool tight) { return 2 * 2 * 2 *
 //       of the C_in channels; K = k k taps x blocks of 64 output channels of
 //       dw^ (the transposed convolution); the epilogue takes dC/dt_in.
 // 128 / Mp positions per tile. Persistent: CTA b takes tiles b, b + grid, ...
-//   warp 0  TMA producer (one lane): A boxes and the B tiles (or, with RES,
-//           every B tile once)
-//   warp 1  TMEM allocation and MMA issue (one lane)
+//   warp 0  TMA producer: A boxes and the B tiles (or, with RES, every B tile
+//           once)
+//   warp 1  TMEM allocation and MMA issue
 //   warps 2-9  epilogue: warp w reads TMEM lane quarter w % 4, 32-column
 //              chunks (w - 2) / 4, +2, ... of the tile
 // ROWBOX (stride 1, tiles within one image row): one box of 128/Mp + k - 1
 // positions per (kh, channel block) serves all k taps kw of that filter row;
 // tap kw's A tile starts kw (FWD) or k - 1 - kw (dS) positions into it.
 // Barriers: full/empty per unit; acc_full/acc_empty per accumulator (two).
+// The two issuing warps run their loops as whole warps (see elect_one): by one
+// lane alone an MMA took about 100 clocks to issue. Forward contraction with
+// the scan, before and after: 128 -> 128 at 14 x 14, B = 256, M = 64: 0.90 ->
+// 0.78 ms; 5x5 128 -> 128 at 8 x 8, B = 50, M = 20: 125 -> 89 us.
 // ---------------------------------------------------------------------------
 template <int BN, bool ROWBOX, bool RES, bool FWD>
 __global__ void __launch_bounds__(CONV_THREADS, 1)
@@ -452,17 +444,18 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
+            const uint32_t lead = tc::elect_one();
             if (RES) {
                 // every (tap, channel block) B tile of the single column tile, once
                 const int nslices = k * k * ncb;
-                tc::mbar_expect_tx(bres_full, (uint32_t)(nslices * BN * 128));
+                tc::mbar_expect_tx_if(lead, bres_full, (uint32_t)(nslices * BN * 128));
                 for (int q = 0; q < nslices; ++q) {
                     const int tap = q / ncb, cb = q - tap * ncb;
-                    tc::tma_load_2d(tc::smem_u32(bres + q * BN * 128), &mapB, bres_full, tap * kc + cb * 64, 0);
+                    tc::tma_load_2d_if(lead, tc::smem_u32(bres + q * BN * 128), &mapB, bres_full, tap * kc + cb * 64, 0);
                 }
             }
-            // one thread issues every copy: the loops below keep its work per
+            // one warp issues every copy: the loops below keep its work per
             // unit to a few additions (positions decoded once per tile, stage
             // and phase counted, taps stepped)
             uint32_t it = 0;  // units issued
@@ -499,37 +492,38 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                 // class coordinates: tap (kh0 + ih ts, kw0 + iw ts) reads output
                 // position (yy + by0 - ih, xx + bx0 - iw)
                 const bool cls_order = pl.ps == a.stride;
-                // the tile's positions read one run of consecutive positions of
-                // a row for every tap (stride 1 forward; dS in stride classes):
-                // one box of ppt positions (mapR) instead of ppt boxes
-                bool run = !ROWBOX && pl.run_ok && ppt > 1 && (FWD ? a.stride == 1 : cls_order);
+                // the tile's positions read one run of positions of a row for
+                // every tap, the layer's stride apart (forward) or consecutive
+                // (dS in stride classes): one box of ppt positions (mapR, at
+                // stride 2 with an element stride) instead of ppt boxes
+                bool run = !ROWBOX && pl.run_ok && ppt > 1 && (FWD || cls_order);
+                const int run_step = FWD ? a.stride : 1;
 #pragma unroll
                 for (int pp = 1; pp < 4; ++pp)
-                    if (pp < ppt) run = run && pb[pp] == pb[0] && pyy[pp] == pyy[0] && pxx[pp] == pxx[0] + pp;
+                    if (pp < ppt) run = run && pb[pp] == pb[0] && pyy[pp] == pyy[0] && pxx[pp] == pxx[0] + pp * run_step;
                 const int by0 = cls_order ? (q.py + a.pad - q.kh0) / pl.ts : 0;
                 const int bx0 = cls_order ? (q.px + a.pad - q.kw0) / pl.ts : 0;
                 const int nkh = ROWBOX ? k : q.nkh, nkw = ROWBOX ? 1 : q.nkw;
                 for (int ih = 0; ih < nkh && ok; ++ih)
                     for (int iw = 0; iw < nkw && ok; ++iw)
                         for (int cb = 0; cb < ncb; ++cb, ++it) {
-                            if (!tc::mbar_wait_spin(&empty[s], ph ^ 1u)) {
-                                conv_set_status(STATUS_TIMEOUT);
+                            if (!tc::mbar_wait_warp(&empty[s], ph ^ 1u)) {
                                 ok = false;
                                 break;
                             }
-                            tc::mbar_expect_tx(&full[s], (uint32_t)(pl.a_bytes + pl.b_bytes));
+                            tc::mbar_expect_tx_if(lead, &full[s], (uint32_t)(pl.a_bytes + pl.b_bytes));
                             const uint32_t st = tc::smem_u32(smem + s * pl.stage);
                             if (ROWBOX) {
                                 // unit (kh, cb): FWD input positions x0 - pad .. of row y0 - pad + kh;
                                 // dS output positions x0 + pad - (k - 1) .. of row y0 + pad - kh
                                 if (FWD)
-                                    tma_load_5d(st, &mapA, &full[s], cb * 64, 0, x0 - a.pad, y0 - a.pad + ih, b0);
+                                    tc::tma_load_5d_if(lead, st, &mapA, &full[s], cb * 64, 0, x0 - a.pad, y0 - a.pad + ih, b0);
                                 else
-                                    tma_load_5d(st, &mapA, &full[s], cb * 64, 0, x0 + a.pad - (k - 1), y0 + a.pad - ih,
+                                    tc::tma_load_5d_if(lead, st, &mapA, &full[s], cb * 64, 0, x0 + a.pad - (k - 1), y0 + a.pad - ih,
                                                 b0);
                                 if (!RES)
                                     for (int kw = 0; kw < k; ++kw)
-                                        tc::tma_load_2d(st + pl.a_bytes + kw * BN * 128, &mapB, &full[s],
+                                        tc::tma_load_2d_if(lead, st + pl.a_bytes + kw * BN * 128, &mapB, &full[s],
                                                         (ih * k + kw) * kc + cb * 64, ct * BN);
                             } else {
                                 const int kh = q.kh0 + ih * pl.ts, kw = q.kw0 + iw * pl.ts;
@@ -549,11 +543,11 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                                         sy = on ? ny / a.stride : -1;
                                         sx = on ? nx / a.stride : 0;
                                     }
-                                    tma_load_5d(st + pp * Mp * 128, run ? &mapR : &mapA, &full[s], cb * 64, 0, sx, sy,
+                                    tc::tma_load_5d_if(lead, st + pp * Mp * 128, run ? &mapR : &mapA, &full[s], cb * 64, 0, sx, sy,
                                                 pb[pp]);
                                 }
                                 if (!RES)
-                                    tc::tma_load_2d(st + pl.a_bytes, &mapB, &full[s], (kh * k + kw) * kc + cb * 64,
+                                    tc::tma_load_2d_if(lead, st + pl.a_bytes, &mapB, &full[s], (kh * k + kw) * kc + cb * 64,
                                                     ct * BN);
                             }
                             if (++s == NST) {
@@ -562,74 +556,69 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                             }
                         }
             }
+            if (!ok && lead) conv_set_status(STATUS_TIMEOUT);
             const uint32_t n_drain = it < (uint32_t)NST ? it : (uint32_t)NST;
             for (uint32_t i = it - n_drain; i < it; ++i) tc::mbar_wait_spin(&full[i % NST], (i / NST) & 1u);
             if (RES) tc::mbar_wait_spin(bres_full, 0);
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(128, BN, false, false);
-            uint32_t j = 0;
-            int s = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            if (RES && !tc::mbar_wait_spin(bres_full, 0)) {
-                conv_set_status(STATUS_TIMEOUT);
-                ok = false;
-            }
-            const int tpu = ROWBOX ? k : 1;  // taps per unit
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++j) {
-                const uint32_t buf = j & 1u;
-                if (j >= 2) {
-                    if (!tc::mbar_wait_spin(&acc_empty[buf], ((j >> 1) + 1u) & 1u)) {
-                        conv_set_status(STATUS_TIMEOUT);
-                        break;
-                    }
-                    tc::tc_fence_after();
+        constexpr uint32_t idesc = idesc_bf16(128, BN, false, false);
+        const uint32_t lead = tc::elect_one();
+        // low descriptor words: stages, resident filters
+        const uint32_t base = tc::sdesc_kk_lo(tc::smem_u32(smem)), bres_lo = tc::sdesc_kk_lo(tc::smem_u32(bres));
+        const uint32_t tmem_u = tc::uniform(tmem);
+        uint32_t j = 0;
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = !RES || tc::mbar_wait_warp(bres_full, 0);
+        const int tpu = ROWBOX ? k : 1;  // taps per unit
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++j) {
+            const uint32_t buf = j & 1u;
+            if (j >= 2) {
+                if (!tc::mbar_wait_warp(&acc_empty[buf], ((j >> 1) + 1u) & 1u)) {
+                    ok = false;
+                    break;
                 }
-                const uint32_t acc = tmem + buf * BN;
-                const DsClass &q = pl.cls[ds_class(pl, t / a.n_col)];
-                const int nkh = ROWBOX ? k : q.nkh, nkw = ROWBOX ? 1 : q.nkw;
-                bool first = true;
-                for (int ih = 0; ih < nkh && ok; ++ih)
-                    for (int iw = 0; iw < nkw && ok; ++iw)
-                        for (int cb = 0; cb < ncb; ++cb) {
-                            if (!tc::mbar_wait_spin(&full[s], ph)) {
-                                conv_set_status(STATUS_TIMEOUT);
-                                ok = false;
-                                break;
-                            }
-                            tc::tc_fence_after();
-                            const uint32_t sa = tc::smem_u32(smem + s * pl.stage);
-                            for (int v = 0; v < tpu; ++v) {
-                                int tap;
-                                uint32_t abase;
-                                if (ROWBOX) {
-                                    tap = ih * k + v;
-                                    abase = sa + (uint32_t)((FWD ? v : k - 1 - v) * Mp * 128);
-                                } else {
-                                    tap = (q.kh0 + ih * pl.ts) * k + q.kw0 + iw * pl.ts;
-                                    abase = sa;
-                                }
-                                const uint32_t bbase = RES ? tc::smem_u32(bres + (tap * ncb + cb) * BN * 128)
-                                                           : sa + (uint32_t)(pl.a_bytes + v * BN * 128);
-                                // descriptors built once; each 16-deep slice is 32 bytes on (+2)
-                                const uint64_t ad = tc::sdesc_sw128(abase), bd = tc::sdesc_sw128(bbase);
-                                tc::mma_bf16(acc, ad, bd, idesc, (!first || v > 0) ? 1u : 0u);
+                tc::tc_fence_after();
+            }
+            const uint32_t acc = tmem_u + buf * BN;
+            const DsClass &q = pl.cls[ds_class(pl, t / a.n_col)];
+            const int nkh = ROWBOX ? k : q.nkh, nkw = ROWBOX ? 1 : q.nkw;
+            uint32_t more = 0;
+            for (int ih = 0; ih < nkh && ok; ++ih)
+                for (int iw = 0; iw < nkw && ok; ++iw)
+                    for (int cb = 0; cb < ncb; ++cb) {
+                        if (!tc::mbar_wait_warp(&full[s], ph)) {
+                            ok = false;
+                            break;
+                        }
+                        tc::tc_fence_after();
+                        const uint32_t st = tc::uniform(base + (uint32_t)(s * (pl.stage >> 4)));
+                        const int tap0 = ROWBOX ? ih * k : (q.kh0 + ih * pl.ts) * k + q.kw0 + iw * pl.ts;
+                        // filters: resident, slices of one channel block ncb apart, or behind the source box
+                        uint32_t blo = RES ? bres_lo + (uint32_t)((tap0 * ncb + cb) * (BN * 8)) : st + (uint32_t)(pl.a_bytes >> 4);
+                        const uint32_t b_step = (uint32_t)((RES ? ncb : 1) * (BN * 8));
+                        uint32_t alo = st + (uint32_t)(ROWBOX && !FWD ? (k - 1) * Mp * 8 : 0);
+                        const uint32_t a_step = (uint32_t)((FWD ? 1 : -1) * Mp * 8);
+                        if (lead) {
+                            for (int v = 0; v < tpu; ++v, alo += a_step, blo += b_step) {
+                                tc::mma_kk(acc, alo, blo, idesc, more | (v > 0 ? 1u : 0u));
 #pragma unroll
-                                for (int kk = 1; kk < 4; ++kk) tc::mma_bf16(acc, ad + 2 * kk, bd + 2 * kk, idesc, 1u);
-                            }
-                            first = false;
-                            tc::mma_commit(&empty[s]);
-                            if (++s == NST) {
-                                s = 0;
-                                ph ^= 1u;
+                                for (int kk = 1; kk < 4; ++kk) tc::mma_kk(acc, alo + 2 * kk, blo + 2 * kk, idesc, 1u);
                             }
                         }
-                if (ok) tc::mma_commit(&acc_full[buf]);
-            }
+                        __syncwarp();
+                        more = 1u;
+                        tc::mma_commit_if(lead, &empty[s]);
+                        if (++s == NST) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
+                    }
+            if (ok) tc::mma_commit_if(lead, &acc_full[buf]);
         }
+        if (!ok && lead) conv_set_status(STATUS_TIMEOUT);
         __syncwarp();
     } else if (FWD) {
         // Scan in the epilogue. Epilogue group g takes the tiles of
@@ -1862,15 +1851,17 @@ static EncodeFn conv_encode() {
 }
 
 // activation [ni][h][w][Mp][C] bf16 as a 5-D map (C, Mp, w, h, ni), boxes of
-// (64, Mp, box_x, 1, 1), 128-byte swizzle, zeros outside
-static bool map_act(CUtensorMap *m, const void *ptr, int ni, int h, int w, int Mp, int C, int box_x = 1) {
+// (64, Mp, box_x, 1, 1) positions every step_x in x, 128-byte swizzle, zeros
+// outside
+static bool map_act(CUtensorMap *m, const void *ptr, int ni, int h, int w, int Mp, int C, int box_x = 1,
+                    int step_x = 1) {
     EncodeFn enc = conv_encode();
-    if (!enc) return false;
+    if (!enc || step_x > 8 || (box_x - 1) * step_x + 1 > 256) return false;
     cuuint64_t dims[5] = {(cuuint64_t)C, (cuuint64_t)Mp, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)ni};
     cuuint64_t strides[4] = {(cuuint64_t)C * 2, (cuuint64_t)Mp * C * 2, (cuuint64_t)w * Mp * C * 2,
                              (cuuint64_t)h * w * Mp * C * 2};
-    cuuint32_t box[5] = {64, (cuuint32_t)Mp, (cuuint32_t)box_x, 1, 1};
-    cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    cuuint32_t box[5] = {64, (cuuint32_t)Mp, (cuuint32_t)((box_x - 1) * step_x + 1), 1, 1};
+    cuuint32_t es[5] = {1, 1, (cuuint32_t)step_x, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(ptr), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -2030,6 +2021,25 @@ static DsPlan tap_plan(int k, int ppt, int Mp, int BN, bool resident, long long 
     return pl;
 }
 
+// dS: row boxes at stride 1 when every tile lies within one image row and two
+// stages fit; resident transposed filters when they are small
+static DsPlan ds_tap_plan(const ConvGeom &g, int C_out, int Mp, bool &resident, bool &rowbox) {
+    const int BN = pick_bn(g.C), ppt = 128 / Mp, ncb = C_out / 64;
+    const long long res = (long long)g.k * g.k * ncb * BN * 128;
+    resident = g.C == BN && res <= 80 * 1024;
+    const bool row_ok = g.s == 1 && g.W % ppt == 0 && ppt + g.k - 1 <= 256;
+    DsPlan pl = tap_plan(g.k, ppt, Mp, BN, resident, res, row_ok, DS_EPI_BYTES, ncb);
+    rowbox = row_ok && pl.nst >= 2;
+    if (!rowbox) pl = tap_plan(g.k, ppt, Mp, BN, resident, res, false, DS_EPI_BYTES, ncb);
+    return pl;
+}
+
+bool conv_ds_row_boxes(const ConvGeom &g, int C_out, int Mp) {
+    bool resident, rowbox;
+    ds_tap_plan(g, C_out, Mp, resident, rowbox);
+    return rowbox;
+}
+
 // dS of ni images with the input-time gradient: dw^ [ni Ho Wo][Mp][C_out],
 // Wt [C_in][k k C_out], t_in [ni H W][C_in] -> g_t_in (zeroed first)
 cudaError_t launch_conv_ds_gemm(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *dW_hat,
@@ -2039,22 +2049,14 @@ cudaError_t launch_conv_ds_gemm(const ConvGeom &g, int ni, int C_out, const LifC
     a.P_rows = ni * g.H * g.W;
     const int BN = pick_bn(g.C);
     const int ppt = 128 / c.Mp;
-    const int ncb = C_out / 64;
     a.n_col = g.C / BN;
     a.t_in = t_in;
     a.g_t_in = g_t_in;
     a.C_t = C_t;
     cudaError_t e = cudaMemsetAsync(g_t_in, 0, sizeof(float) * (size_t)a.P_rows * C_t, st);
     if (e != cudaSuccess) return e;
-    // resident transposed filters when they are small; one box per filter row
-    // at stride 1 when every tile lies within one image row
-    const long long res = (long long)g.k * g.k * ncb * BN * 128;
-    const bool resident = a.n_col == 1 && res <= 80 * 1024;
-    auto plan = [&](bool rowbox) { return tap_plan(g.k, ppt, c.Mp, BN, resident, res, rowbox, DS_EPI_BYTES, ncb); };
-    const bool row_ok = g.s == 1 && g.W % ppt == 0 && ppt + g.k - 1 <= 256;
-    DsPlan pl = plan(row_ok);
-    bool rowbox = row_ok && pl.nst >= 2;
-    if (!rowbox) pl = plan(false);
+    bool resident, rowbox;
+    DsPlan pl = ds_tap_plan(g, C_out, c.Mp, resident, rowbox);
     if (pl.nst < 2) return cudaErrorInvalidConfiguration;
     // stride classes (one for stride 1); a stride whose s x s classes do not
     // fit runs every tap in the identity order, off-grid taps reading zeros
@@ -2173,7 +2175,7 @@ cudaError_t launch_conv_fwd_tma(const ConvGeom &g, int ni, int C_out, const LifC
     if (!map_act(&mA, S, ni, g.H, g.W, c.Mp, g.C, rowbox ? ppt + g.k - 1 : 1) ||
         !map_mat(&mB, Wf, C_out, g.k * g.k * g.C, BN))
         return cudaErrorInvalidValue;
-    pl.run_ok = map_act(&mR, S, ni, g.H, g.W, c.Mp, g.C, ppt) ? 1 : 0;
+    pl.run_ok = map_act(&mR, S, ni, g.H, g.W, c.Mp, g.C, ppt, g.s) ? 1 : 0;
     if (!pl.run_ok) mR = mA;
 #define DSTD_FT(BNV)                                                                                   \
     if (rowbox) return resident ? launch_tap_bn<BNV, true, true, true>(mA, mB, mR, a, pl, st)          \

@@ -2,11 +2,10 @@
 (operand policy 2, whose results the conv parity tests hold to the oracle).
 
 Forward: the same products in the same order per output, so spike times and saved state are equal bit for bit.
-Input-time gradient: the same products, in another order where a filter row has several channel blocks and the
-stride is 2; at most K / 16 = 225 fp32 accumulations of 2^-24 each per sum, 1.4e-5 relative to the sum of the terms'
-magnitudes, of which independent signs leave a small part: 2e-5 relative L2.
+Input-time gradient: the same products in the same order too; the two bins of an input may be added in either order.
+Weight gradient: fp32 sums in another order, at most a few hundred accumulations of 2^-24 each: 2e-5 relative L2.
 Shapes: widths that the position tile does not divide, odd grids at stride 2, one image row, 1x1, 5x5 and 7x7
-filters, filters resident and streamed, several column tiles and channel blocks, padded input channels, chunks."""
+filters, filters resident and streamed, several channel blocks, padded input channels, chunks."""
 
 import math
 
@@ -65,31 +64,38 @@ def rel(a, b):
     return float((a - b).norm() / b.norm().clamp(min=1e-30))
 
 
-# B, H, W, C_in, C_out, k, stride, pad, M, tau
+# H, W, C_in, C_out, k, stride, pad, M, tau; the batch is taken just large enough for the row kernels to be chosen
 CASES = [
-    (2, 28, 28, 64, 64, 3, 1, 1, 64, (1.0, 0.25)),
-    (3, 7, 7, 64, 64, 3, 1, 1, 50, (0.5, 0.25)),        # odd width, M below the padded 64
-    (2, 5, 9, 64, 64, 3, 1, 1, 20, (INF, INF)),         # rows and columns differ, four positions per tile
-    (1, 1, 6, 64, 64, 3, 1, 1, 32, (INF, INF)),         # one image row
-    (2, 6, 6, 3, 64, 3, 1, 1, 32, (INF, INF)),          # padded input channels
-    (2, 9, 9, 64, 128, 3, 2, 1, 64, (1.0, 0.25)),       # stride 2 on an odd grid
-    (2, 8, 8, 64, 128, 3, 2, 1, 33, (0.4, 0.2)),        # and on an even one
-    (2, 10, 10, 128, 64, 3, 2, 1, 32, (INF, INF)),      # stride 2, two channel blocks
-    (2, 14, 14, 128, 128, 3, 1, 1, 64, (1.0, 0.25)),    # streamed filters, two channel blocks
-    (2, 8, 8, 128, 256, 3, 1, 1, 32, (INF, INF)),       # two column tiles
-    (2, 7, 7, 256, 64, 3, 1, 1, 32, (0.5, 0.25)),       # four channel blocks, width 7
-    (2, 8, 8, 128, 128, 5, 1, 2, 20, (INF, INF)),       # 5x5
-    (2, 8, 8, 64, 64, 1, 1, 0, 32, (INF, INF)),         # 1x1
-    (2, 9, 9, 64, 64, 7, 1, 3, 32, (0.5, 0.25)),        # 7x7
-    (2, 9, 9, 64, 64, 5, 2, 2, 64, (0.5, 0.25)),        # 5x5 at stride 2
-    (2, 8, 8, 64, 64, 3, 1, 0, 32, (INF, INF)),         # no padding
-    (2, 8, 8, 64, 64, 3, 1, 2, 32, (INF, INF)),         # padding k - 1
+    (28, 28, 64, 64, 3, 1, 1, 64, (1.0, 0.25)),
+    (7, 7, 64, 64, 3, 1, 1, 50, (0.5, 0.25)),        # odd width, M below the padded 64
+    (5, 9, 64, 64, 3, 1, 1, 20, (INF, INF)),         # rows and columns differ, four positions per tile
+    (1, 6, 64, 64, 3, 1, 1, 32, (INF, INF)),         # one image row
+    (6, 6, 3, 64, 3, 1, 1, 32, (INF, INF)),          # padded input channels
+    (9, 9, 64, 128, 3, 2, 1, 64, (1.0, 0.25)),       # stride 2 on an odd grid, two channel blocks in dS
+    (8, 8, 64, 128, 3, 2, 1, 33, (0.4, 0.2)),        # and on an even one
+    (10, 10, 64, 64, 3, 2, 1, 32, (INF, INF)),       # stride 2, one channel block
+    (14, 14, 64, 128, 3, 1, 1, 64, (1.0, 0.25)),     # two channel blocks in dS
+    (7, 7, 64, 256, 3, 1, 1, 32, (0.5, 0.25)),       # four, at a width that the tile does not divide
+    (8, 8, 64, 64, 5, 1, 2, 20, (INF, INF)),         # 5x5
+    (8, 8, 64, 64, 1, 1, 0, 32, (INF, INF)),         # 1x1
+    (9, 9, 64, 64, 7, 1, 3, 32, (0.5, 0.25)),        # 7x7
+    (9, 9, 64, 64, 5, 2, 2, 64, (0.5, 0.25)),        # 5x5 at stride 2
+    (8, 8, 64, 64, 3, 1, 0, 32, (INF, INF)),         # no padding
+    (8, 8, 64, 64, 3, 1, 2, 32, (INF, INF)),         # padding k - 1
 ]
 
 
-@pytest.mark.parametrize("case", CASES, ids=lambda c: "-".join(str(x) for x in c[:9]))
+def batch(case):
+    Ho, Wo = ((case[i] + 2 * case[6] - case[4]) // case[5] + 1 for i in (0, 1))
+    # forward: 300 output positions per SM; dS alone (more than 64 output channels or stride 2): 20 input positions
+    need = 300 * 152 // (Ho * Wo) if case[3] == 64 and case[5] == 1 else 20 * 152 // (case[0] * case[1])
+    return need + 1
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "-".join(str(x) for x in c[:8]))
 def test_rows_match_one_row_at_a_time(case):
-    a, b = run(*case, policy=0), run(*case, policy=2)
+    B = batch(case)
+    a, b = run(B, *case, policy=0), run(B, *case, policy=2)
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
     assert torch.isfinite(a[0]).any()
     assert rel(a[2], b[2]) <= 1e-5
@@ -98,7 +104,8 @@ def test_rows_match_one_row_at_a_time(case):
 
 
 def test_rows_chunks_agree():
-    case = (5, 6, 6, 64, 64, 3, 1, 1, 32, (INF, INF))
-    a, b = run(*case, policy=0), run(*case, policy=0, chunk=2)
+    case = (6, 6, 64, 64, 3, 1, 1, 32, (INF, INF))
+    B = batch(case)
+    a, b = run(2 * B, *case, policy=0), run(2 * B, *case, policy=0, chunk=B)
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and torch.equal(a[3], b[3])
     assert rel(a[4], b[4]) <= 2e-5
