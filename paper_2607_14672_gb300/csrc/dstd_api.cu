@@ -1069,8 +1069,11 @@ int dstd_dense_bwd(const float *t_in, const float *W, const float *t_out, const 
         a.bw = ws.bw;
         Timed tm(KK_GEMM_DS, st);
         // dw^ read transposed from its dW layout [N_out, B*Mp]
-        TRY(cu(launch_tc_gemm(ws.wt_hi, ws.wt_lo, ws.ldt, ws.dA_hi, ws.dA_lo, ws.ldbm, N_in, (int)cols, N_out, 1, op,
-                              Epi::GradT, a, st, true)));
+        if (op == OpKind::BF16 && tc_gemm_pair_preferred(N_in, (int)cols, N_out, op))
+            TRY(cu(launch_tc_gemm_pair_gradt(ws.wt_hi, ws.ldt, ws.dA_hi, ws.ldbm, N_in, (int)cols, N_out, a, st)));
+        else
+            TRY(cu(launch_tc_gemm(ws.wt_hi, ws.wt_lo, ws.ldt, ws.dA_hi, ws.dA_lo, ws.ldbm, N_in, (int)cols, N_out, 1,
+                                  op, Epi::GradT, a, st, true)));
     }
     if (dw_on_pairs(N_in, N_out, (int)cols, op)) {
         // on SM pairs, computed transposed: (s^T dw^)[j, i] stored as dW[i][j];

@@ -436,7 +436,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 //   empty[s]   in both CTAs, released by the even CTA's MMA commit (multicast);
 //   acc_full   in both CTAs, by the same commit after a tile's last MMA;
 //   acc_empty  the even CTA's, arrived on by the epilogue warps of both.
-// Epilogue StoreT: D^T[c][r] = acc[r][c] * col_scale[c], the transposed
+// Epilogues: GradT, the dS contraction of the bf16 mode (B MN-major as in the
+// single-CTA kernel; 16384 wide, M = 128: 6.7 -> 5.5 ms), and StoreT: D^T[c][r] = acc[r][c] * col_scale[c], the transposed
 // store (the forward computes w^ as S W^T: rows (b, m), columns i, written
 // as w^[i][(b, m)]; consecutive lanes, consecutive addresses).
 // Every wait is bounded; neither CTA leaves before the other (cluster
@@ -562,13 +563,14 @@ __device__ __forceinline__ void mma_pair_kk(uint32_t d_tmem, uint32_t alo, uint3
         : "memory");
 }
 
-template <int NPASS, bool F16>
+template <int NPASS, bool F16, int EPI, bool BMN>
 __global__ void __launch_bounds__(pair_threads<NPASS>(), 1)
     k_tc_gemm_pair(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ CUtensorMap mA_lo,
                    const __grid_constant__ CUtensorMap mB_hi, const __grid_constant__ CUtensorMap mB_lo, int R,
                    int Cn, int ktiles, int n_row, int n_col, TcEpiArgs args) {
     using C = Cfg2<NPASS>;
     constexpr int MW = pair_mma_warps<NPASS>();
+    static_assert(!BMN || NPASS == 1, "the MN-major B of the pair kernel: bf16 mode only");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + C::STAGES * C::STAGE);
@@ -626,7 +628,8 @@ __global__ void __launch_bounds__(pair_threads<NPASS>(), 1)
                     tma_load_2d_pair(st, &mA_hi, fb, kx, row0);
                     if (NPASS == 3) tma_load_2d_pair(st + C::A_BYTES, &mA_lo, fb, kx, row0);
                     const uint32_t sb = st + C::NOP * C::A_BYTES;
-                    tma_load_2d_pair(sb, &mB_hi, fb, kx, brow0);
+                    if (BMN) tma_load_2d_pair(sb, &mB_hi, fb, brow0, kx);  // 64 rows of k, this CTA's 64 columns
+                    else tma_load_2d_pair(sb, &mB_hi, fb, kx, brow0);
                     if (NPASS == 3) tma_load_2d_pair(sb + C::B_BYTES, &mB_lo, fb, kx, brow0);
                 }
             }
@@ -653,7 +656,7 @@ __global__ void __launch_bounds__(pair_threads<NPASS>(), 1)
             // each) cover them. Every warp passes every stage, so that none is
             // ever two barrier phases off. 16384 wide, M = 128: forward and
             // dW 7.1 -> 5.2 ms each, 0.87 of the measured peak.
-            constexpr uint32_t idesc = idesc_16bit(2 * BM2, C::BNP, F16);
+            constexpr uint32_t idesc = idesc_16bit(2 * BM2, C::BNP, F16, BMN);
             const uint32_t lead = elect_one(), mw = (uint32_t)(warp - 1);
             const uint32_t base = sdesc_kk_lo(smem_u32(smem)), tmem_u = uniform(tmem);
             uint32_t it = 0, j = 0;
@@ -682,7 +685,7 @@ __global__ void __launch_bounds__(pair_threads<NPASS>(), 1)
                         if (lead) {
 #pragma unroll
                             for (int kk = 0; kk < BK / 16; ++kk)
-                                mma_pair_kk(acc, alo + 2 * kk, blo + 2 * kk, idesc, kk > 0 ? 1u : more);
+                                mma_pair_kk(acc, alo + 2 * kk, blo + (BMN ? 128 : 2) * kk, idesc, kk > 0 ? 1u : more);
                         }
                         __syncwarp();
                     }
@@ -751,26 +754,57 @@ __global__ void __launch_bounds__(pair_threads<NPASS>(), 1)
         const int quarter = warp & 3, group = ew >> 2;
         const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16);
         const uint32_t acc_empty0 = mapa_rank(smem_u32(acc_empty), 0);
-        const int c_lo = group * GCOLS;
         const int n_main = ktiles < C::P_MAIN ? ktiles : C::P_MAIN;
+        // columns of a group: GCOLS, or (GradT) a whole sample when one spans more
+        const int span = (EPI == (int)Epi::GradT && args.c.Mp > GCOLS) ? args.c.Mp : GCOLS;
+        int c_lo = group * span, c_hi = c_lo + span;
+        if (c_lo >= C::BNP) c_lo = c_hi = C::BNP;
+        if (c_hi > C::BNP) c_hi = C::BNP;
         uint32_t j = 0;
         for (int t = cid; t < ntiles; t += ncl, ++j) {
             int rt, ct;
             tile_order(t, n_row, n_col, BAND_PAIR, rt, ct);
             const int row = rt * (2 * BM2) + rank * BM2 + quarter * 32 + lane;
-            const int col0 = ct * C::BNP + c_lo;
+            const int col0 = ct * C::BNP + (EPI == (int)Epi::Store ? c_lo : 0);
             if (!mbar_wait_cluster(acc_full, j & 1u, true)) {
                 set_status(STATUS_TIMEOUT);
                 break;
             }
             tc_fence_after();
+            if (EPI == (int)Epi::GradT && c_hi - c_lo != GCOLS) {
+                // a sample spans more than GCOLS columns, or the group is idle
+                BinW w{-100, 0.f, 0.f, 0.f, 0.f};
+                float g = 0.f;
+                for (int cc = c_lo; cc < c_hi; cc += 32) {
+                    float v[32];
+                    tmem_ld_acc<C::BNP>(tbase, cc, n_main, NPASS == 3, v);
+                    gradt_chunk<32>(v, row, col0 + cc, w, g, args);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(acc_empty0);
+                continue;
+            }
             float v[GCOLS / 32][32];
 #pragma unroll
             for (int h = 0; h < GCOLS / 32; ++h) tmem_ld_acc<C::BNP>(tbase, c_lo + 32 * h, n_main, NPASS == 3, v[h]);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(acc_empty0);
-            if (row < R) {
+            if (EPI == (int)Epi::GradT) {
+                BinW w{-100, 0.f, 0.f, 0.f, 0.f};
+                float g = 0.f;
+                if (args.c.Mp == 8) {
+#pragma unroll
+                    for (int h = 0; h < GCOLS / 32; ++h) gradt_chunk<8>(v[h], row, col0 + c_lo + 32 * h, w, g, args);
+                } else if (args.c.Mp == 16) {
+#pragma unroll
+                    for (int h = 0; h < GCOLS / 32; ++h) gradt_chunk<16>(v[h], row, col0 + c_lo + 32 * h, w, g, args);
+                } else {
+#pragma unroll
+                    for (int h = 0; h < GCOLS / 32; ++h) gradt_chunk<32>(v[h], row, col0 + c_lo + 32 * h, w, g, args);
+                }
+            } else if (row < R) {
 #pragma unroll
                 for (int h = 0; h < GCOLS / 32; ++h) {
 #pragma unroll
@@ -866,12 +900,12 @@ cudaError_t launch_wait_selftest(unsigned long long limit_ns, cudaStream_t st) {
 namespace tc {
 // SM pairs that can hold a pair kernel's clusters at once (a pair must sit in
 // one GPC: a GPC with an odd number of usable SMs leaves one out)
-template <int NPASS, bool F16>
+template <int NPASS, bool F16, int EPI = 0, bool BMN = false>
 static int resident_pairs() {
     static int resident = 0;
     if (resident == 0) {
         using C = Cfg2<NPASS>;
-        auto kern = k_tc_gemm_pair<NPASS, F16>;
+        auto kern = k_tc_gemm_pair<NPASS, F16, EPI, BMN>;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess) return 0;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
@@ -891,12 +925,12 @@ static int resident_pairs() {
     return resident;
 }
 
-template <int NPASS, bool F16>
+template <int NPASS, bool F16, int EPI = 0, bool BMN = false>
 static cudaError_t launch_pair(const CUtensorMap &a_hi, const CUtensorMap &a_lo, const CUtensorMap &b_hi,
                                const CUtensorMap &b_lo, int R, int Cn, int K, const TcEpiArgs &args,
                                cudaStream_t st) {
     using C = Cfg2<NPASS>;
-    auto kern = k_tc_gemm_pair<NPASS, F16>;
+    auto kern = k_tc_gemm_pair<NPASS, F16, EPI, BMN>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     const int ktiles = (K + BK - 1) / BK;
@@ -914,7 +948,7 @@ static cudaError_t launch_pair(const CUtensorMap &a_hi, const CUtensorMap &a_lo,
     cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = st;
     // persistent: as many pairs as can be resident at once
-    const int resident = resident_pairs<NPASS, F16>();
+    const int resident = resident_pairs<NPASS, F16, EPI, BMN>();
     if (resident < 1) return cudaErrorInvalidConfiguration;
     const int pairs = (int)(ntiles < resident ? ntiles : resident);
     cfg.gridDim = dim3(2 * pairs);
@@ -974,6 +1008,14 @@ cudaError_t launch_tc_gemm_pair_storeT(const void *A_hi, const void *A_lo, int l
     a_lo = a_hi;
     b_lo = b_hi;
     return tc::launch_pair<1, false>(a_hi, a_lo, b_hi, b_lo, R, Cn, K, args, st);
+}
+
+cudaError_t launch_tc_gemm_pair_gradt(const void *A, int lda, const void *B, int ldb, int R, int Cn, int K,
+                                      const TcEpiArgs &args, cudaStream_t st) {
+    CUtensorMap a, b;
+    if (!tc::make_map(&a, A, R, K, lda, tc::BM2, false) || !tc::make_map(&b, B, K, Cn, ldb, tc::BK, false))
+        return cudaErrorInvalidValue;
+    return tc::launch_pair<1, false, (int)Epi::GradT, true>(a, a, b, b, R, Cn, K, args, st);
 }
 
 int tc_gemm_splits_valid(int K, int splits) {

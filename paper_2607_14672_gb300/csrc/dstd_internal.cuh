@@ -649,6 +649,10 @@ cudaError_t launch_tc_gemm(const void *A_hi, const void *A_lo, int lda, const vo
 cudaError_t launch_tc_gemm_pair_storeT(const void *A_hi, const void *A_lo, int lda, const void *B_hi, const void *B_lo,
                                        int ldb, int R, int Cn, int K, OpKind op, const TcEpiArgs &args,
                                        cudaStream_t st);
+// The GradT contraction of launch_tc_gemm on SM pairs, bf16 operands: A [R, K]
+// rows, B [K, Cn] rows; the same results bit for bit.
+cudaError_t launch_tc_gemm_pair_gradt(const void *A, int lda, const void *B, int ldb, int R, int Cn, int K,
+                                      const TcEpiArgs &args, cudaStream_t st);
 // whether the pair kernel is expected to beat the single-CTA one for an
 // R x Cn x K product (resident pairs counted once per process)
 bool tc_gemm_pair_preferred(int R, int Cn, int K, OpKind op);

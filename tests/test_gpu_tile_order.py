@@ -1,4 +1,4 @@
-"""Order of the dense contraction's output tiles: bands of 12 row tiles (128 rows each) on single CTAs, of 6
+"""The dense contraction's kernels against each other and the oracle. Order of the output tiles: bands of 12 row tiles (128 rows each) on single CTAs, of 6
 (256 rows) on SM pairs. Shapes whose last band is partial, in both operand modes and on both kernels, against the
 oracle's w^ within the bound of the contraction's own parity test."""
 
@@ -55,3 +55,32 @@ def test_partial_band(math_mode, policy, B, N_in, N_out):
         bound = bound + 3e-5 * prod(np.abs(s), aW)
     err = np.abs(what.cpu().numpy().astype(np.float64) - ref)
     assert (err <= bound).all(), float(np.max(err / bound))
+
+
+@pytest.mark.parametrize("B,N_in,N_out,M", [(9, 300, 140, 8), (5, 257, 70, 16), (4, 520, 200, 20), (3, 200, 300, 50),
+                                            (2, 513, 333, 100), (64, 1700, 72, 32), (1, 8, 129, 128)])
+def test_input_gradient_on_pairs(B, N_in, N_out, M):
+    """bf16 dS with the input-time gradient in its epilogue: SM pairs and single CTAs add in the same order per
+    accumulator, so the gradient is equal bit for bit (every padded grid size, ragged rows and columns)."""
+    from paper_2607_14672_gb300 import dstd
+    t_in, layer = dense_layer(B, N_in, N_out, M, 0.5, 0.25, seed=N_in + M, t_offset=0.001, fire=0.6)
+    p = dstd.params(layer, 1.0 / B)
+    dev = lambda x: torch.tensor(np.asarray(x), dtype=torch.float32, device="cuda").contiguous()
+    t, W = dev(t_in), dev(layer["W"])
+    up = dev(np.random.default_rng(M).normal(size=(B, N_out)))
+    ws = torch.empty(dstd.dense_workspace_bytes(B, N_in, N_out, p, "bf16"), dtype=torch.uint8, device="cuda")
+    out = torch.empty(B, N_out, device="cuda")
+    saved = torch.empty(dstd.dense_saved_bytes(B, N_out), dtype=torch.uint8, device="cuda")
+    dstd.dense_fwd(t, W, p, "bf16", out, saved, torch.empty(4, device="cuda"), ws)
+    got = []
+    for policy in (1, 2):
+        g_in, g_W = torch.full_like(t, 7.0), torch.empty_like(W)
+        prev = dstd.set_pair_policy(policy)
+        try:
+            dstd.dense_bwd(t, W, out, saved, up, p, "bf16", g_in, g_W, ws)
+            torch.cuda.synchronize()
+        finally:
+            dstd.set_pair_policy(prev)
+        got.append(g_in)
+    assert torch.isfinite(out).any() and (got[0] != 0).any()
+    assert torch.equal(got[0], got[1])
