@@ -825,7 +825,10 @@ int conv_bwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
                 TRY(cu(launch_bin_rec(t_in + in_off, (long long)ni * g.H * g.W * g.C, c, ws.rec, st)));
         }
         Timed tm(KK_GEMM_DW, st);
-        if (ws.S)
+        if (ws.S && g_conv_operand_policy == 0 && conv_dw_cols_supported(gp, C_out, Mp))
+            TRY(cu(launch_conv_dw_cols(gp, ni, C_out, c, ws.S, ws.dwh, last ? ws.count : nullptr, qcoef, g_W, g.C,
+                                       st)));
+        else if (ws.S)
             TRY(cu(launch_conv_dw_tma(gp, ni, C_out, c, ws.S, ws.dwh, last ? ws.count : nullptr, qcoef, g_W, g.C,
                                       st)));
         else

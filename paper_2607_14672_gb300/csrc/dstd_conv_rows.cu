@@ -1,5 +1,5 @@
-// Conv forward and dS contractions on sm_103a that take each row of the source
-// image once (tcgen05, bf16 operands, fp32 accumulation).
+// Conv contractions on sm_103a that take each part of their source image once:
+// forward and dS by rows (tcgen05, bf16 operands, fp32 accumulation).
 //
 // A work item is a run of output rows of one image, one tile of output
 // positions wide (ppt = 128 / Mp positions per 128-row MMA tile, NT tiles) and
@@ -26,6 +26,9 @@
 // one-row-at-a-time kernels: filter row, then (channel block, filter column)
 // or (filter column, channel block) as those take them for the same shape, so
 // both give the same w^.
+//
+// dW of 3x3 layers at stride 1 (k_conv_dw_cols) reads each column of the binned
+// input once in the same spirit.
 //
 // Every mbarrier wait is bounded; an expired wait sets this unit's status
 // word, the role stops, and the CTA still frees its TMEM.
@@ -914,6 +917,239 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
 }
 
 // ---------------------------------------------------------------------------
+// dW of 3x3 layers at stride 1, walking the output rows position by position:
+//   dW[o, (kh, kw), c] = sum_{y, x, m} dw^[(y, x, m), o] S[(y + kh, x + kw, m), c]
+// A K step is one output position (Mp grid steps). Its nine taps read three
+// columns of S, two of which the step before has read: a ring of columns in
+// shared memory (the S boxes of the rows y - pad .. for one x, one copy each,
+// and the dw^ box of the position that the column completes) is filled once
+// per position where a box per tap and position was loaded before: 32 KB
+// instead of 88 KB per step (64 channels, Mp = 64), with three and more
+// columns in flight instead of one step.
+// The filter rows of the layer's channel block form 128-row MMA blocks: the
+// taps (0, kw) and (1, kw) together (their boxes lie side by side), tap
+// (2, kw) alone (the other 64 rows of the block are not used); with 64 output
+// channels per tile all six blocks share a CTA, with 128 the first three and
+// the last three are tiles of their own (TMEM holds four accumulators of 128
+// columns). Split over output rows; fp32 atomics into g_W. Warps: 0 TMA, 1-4
+// MMA issue (block b by warp b mod 4), 5-12 epilogue. Bound by the MMAs' reads
+// of shared memory. Measured, a box per tap before and by columns (B = 256,
+// M = 64): 64 -> 64 at 28 x 28 1.29 -> 0.90 ms, 128 -> 128 at 14 x 14
+// 0.79 -> 0.57 ms.
+// ---------------------------------------------------------------------------
+constexpr int DWC_MAX_RING = 8;
+constexpr int DWC_MMA_WARPS = 4;
+constexpr int DWC_THREADS = (1 + DWC_MMA_WARPS + 8) * 32;
+
+struct DwColsPlan {
+    int Ho, Wo, pad, Mp, ncb, n_col;
+    int rows, rows_per, n_tiles, ring;
+    int C_t;              // the layer's input channels (below 64: padded to 64 in S)
+    float *g_W;           // [C_out][9][C_t]
+    const float *count;   // silent neurons per output channel, or null
+    float qcoef;
+};
+
+template <int BN>
+__global__ void __launch_bounds__(DWC_THREADS, 1)
+    k_conv_dw_cols(const __grid_constant__ CUtensorMap mapS0, const __grid_constant__ CUtensorMap mapS1,
+                   const __grid_constant__ CUtensorMap mapD, const __grid_constant__ DwColsPlan p) {
+    constexpr int NGRP = BN == 64 ? 1 : 2;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int box = p.Mp * 128;
+    const int slot_bytes = ((NGRP == 1 ? 3 : 2) + BN / 64) * box;  // (the second group's slots are one box smaller)
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + p.ring * slot_bytes);
+    uint64_t *empty = full + DWC_MAX_RING;
+    uint64_t *acc_full = empty + DWC_MAX_RING;
+    uint64_t *acc_empty = acc_full + 1;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int per = p.ncb * NGRP * p.n_col;  // tiles of one range of rows
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < DWC_MAX_RING; ++s) {
+            tc::mbar_init(&full[s], 1);
+            tc::mbar_init(&empty[s], DWC_MMA_WARPS);
+        }
+        tc::mbar_init(acc_full, DWC_MMA_WARPS);
+        tc::mbar_init(acc_empty, 8);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) tc::tmem_alloc(tmem_slot, 512);
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    // tile t: rows [r0, r1) of the (image, y) rows, channel block, group, column tile
+    auto decode = [&](int t, int &r0, int &r1, int &cb, int &grp, int &ct) {
+        const int sp = t / per;
+        int q = t - sp * per;
+        ct = q % p.n_col;
+        q /= p.n_col;
+        grp = q % NGRP;
+        cb = q / NGRP;
+        r0 = sp * p.rows_per;
+        r1 = r0 + p.rows_per < p.rows ? r0 + p.rows_per : p.rows;
+    };
+
+    if (warp == 0) {
+        const uint32_t lead = tc::elect_one();
+        uint32_t n = 0;
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
+            int r0, r1, cb, grp, ct;
+            decode(t, r0, r1, cb, grp, ct);
+            const int nbox = NGRP == 1 ? 3 : 2 - grp, kh0 = NGRP == 1 ? 0 : 2 * grp;
+            int b = r0 / p.Ho, y = r0 - b * p.Ho;
+            for (int r = r0; r < r1 && ok; ++r) {
+                for (int cx = 0; cx < p.Wo + 2; ++cx, ++n) {
+                    if (!tc::mbar_wait_warp(&empty[s], ph ^ 1u)) {
+                        ok = false;
+                        break;
+                    }
+                    // columns 0 and 1 complete no position
+                    tc::mbar_expect_tx_if(lead, &full[s], (uint32_t)((nbox + (cx >= 2 ? BN / 64 : 0)) * box));
+                    const uint32_t st = tc::smem_u32(smem + s * slot_bytes);
+                    tc::tma_load_5d_if(lead, st, grp == 0 ? &mapS0 : &mapS1, &full[s], cb * 64, 0, cx - p.pad,
+                                       y - p.pad + kh0, b);
+                    if (cx >= 2)
+#pragma unroll
+                        for (int h = 0; h < BN / 64; ++h)
+                            tc::tma_load_5d_if(lead, st + (uint32_t)((nbox + h) * box), &mapD, &full[s],
+                                               ct * BN + h * 64, 0, cx - 2, y, b);
+                    if (++s == p.ring) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (++y == p.Ho) {
+                    y = 0;
+                    ++b;
+                }
+            }
+        }
+        if (!ok && lead) rows_set_status(STATUS_TIMEOUT);
+        const uint32_t tail = n < (uint32_t)p.ring ? n : (uint32_t)p.ring;
+        for (uint32_t i = n - tail; i < n; ++i) tc::mbar_wait_spin(&full[i % p.ring], (i / p.ring) & 1u);
+        __syncwarp();
+    } else if (warp <= DWC_MMA_WARPS) {
+        const int mw = warp - 1;
+        const uint32_t lead = tc::elect_one();
+        constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                                   ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);  // both MN-major
+        // low descriptor words: the next 64 columns (of A or of N) one box on
+        const uint32_t base = ((tc::smem_u32(smem) & 0x3FFFFu) >> 4) | ((uint32_t)(box >> 4) << 16);
+        const uint32_t tmem_u = tc::uniform(tmem);
+        const int nkk = p.Mp >> 4;
+        uint32_t j = 0;
+        int s = 0;  // slot of the current column
+        uint32_t ph = 0;
+        bool ok = true;
+        auto back = [&](int q, int d) { return q - d < 0 ? q - d + p.ring : q - d; };
+        for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x, ++j) {
+            int r0, r1, cb, grp, ct;
+            decode(t, r0, r1, cb, grp, ct);
+            const int nbox = NGRP == 1 ? 3 : 2 - grp;
+            constexpr int NBLK = NGRP == 1 ? 6 : 3;
+            if (j >= 1) {
+                if (!tc::mbar_wait_warp(acc_empty, (j - 1) & 1u)) {
+                    ok = false;
+                    break;
+                }
+                tc::tc_fence_after();
+            }
+            uint32_t more = 0;
+            for (int r = r0; r < r1 && ok; ++r) {
+                for (int cx = 0; cx < p.Wo + 2; ++cx) {
+                    if (!tc::mbar_wait_warp(&full[s], ph)) {
+                        ok = false;
+                        break;
+                    }
+                    if (cx >= 2) {
+                        tc::tc_fence_after();
+                        const uint32_t cols =
+                            tc::uniform((uint32_t)(back(s, 2) | (back(s, 1) << 8) | (s << 16)));  // slots of kw = 0, 1, 2
+                        if (lead) {
+                            const uint32_t blo = base + ((cols >> 16) * (uint32_t)slot_bytes + (uint32_t)(nbox * box)) / 16u;
+                            for (int bk = mw; bk < NBLK; bk += DWC_MMA_WARPS) {
+                                const int kw = bk < 3 ? bk : bk - 3, bx = bk < 3 ? 0 : 2;
+                                const uint32_t alo =
+                                    base + (((cols >> (8 * kw)) & 0xffu) * (uint32_t)slot_bytes + (uint32_t)(bx * box)) / 16u;
+                                const uint32_t acc = tmem_u + (uint32_t)(bk * BN);
+                                for (int kk = 0; kk < nkk; ++kk)
+                                    tc::mma_kk(acc, alo + (uint32_t)(kk * 128), blo + (uint32_t)(kk * 128), idesc,
+                                               kk > 0 ? 1u : more);
+                            }
+                        }
+                        __syncwarp();
+                        more = 1u;
+                        tc::mma_commit_if(lead, &empty[back(s, 2)]);
+                        if (cx == p.Wo + 1) {  // the row's last position
+                            tc::mma_commit_if(lead, &empty[back(s, 1)]);
+                            tc::mma_commit_if(lead, &empty[s]);
+                        }
+                    }
+                    if (++s == p.ring) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+            }
+            if (ok) tc::mma_commit_if(lead, acc_full);
+        }
+        if (!ok && lead) rows_set_status(STATUS_TIMEOUT);
+        __syncwarp();
+    } else {
+        const int quarter = warp & 3, half = (warp - 1 - DWC_MMA_WARPS) >> 2;
+        const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
+        const int r = quarter * 32 + lane;
+        uint32_t j = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < p.n_tiles; t += gridDim.x, ++j) {
+            int r0, r1, cb, grp, ct;
+            decode(t, r0, r1, cb, grp, ct);
+            if (__any_sync(0xffffffffu, !tc::mbar_wait_sleep(acc_full, j & 1u))) {
+                ok = false;
+                break;
+            }
+            tc::tc_fence_after();
+            constexpr int NBLK = NGRP == 1 ? 6 : 3;
+            for (int bk = 0; bk < NBLK; ++bk) {
+                const bool pair = NGRP == 1 ? bk < 3 : grp == 0;
+                const int kw = bk < 3 ? bk : bk - 3, kh = pair ? r >> 6 : 2;
+                const int ch = cb * 64 + (r & 63);
+                const bool on = (pair || r < 64) && ch < p.C_t;
+                const long long k0 = (long long)(kh * 3 + kw) * p.C_t + ch;
+                for (int cc = half; cc < BN / 32; cc += 2) {
+                    float v[32];
+                    tc::tmem_ld32(tmem + lane_base + bk * BN + cc * 32, v);
+                    if (on) {
+                        const int o0 = ct * BN + cc * 32;
+#pragma unroll
+                        for (int u = 0; u < 32; ++u) {
+                            const float add = r0 == 0 && p.count ? p.qcoef * p.count[o0 + u] : 0.f;
+                            atomicAdd(p.g_W + (long long)(o0 + u) * 9 * p.C_t + k0, v[u] + add);
+                        }
+                    }
+                }
+            }
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(acc_empty);
+        }
+        if (!ok) rows_set_status(STATUS_TIMEOUT);
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tc::tmem_dealloc(tmem, 512);
+}
+
+// ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
 typedef CUresult (*RowsEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -934,14 +1170,14 @@ RowsEncodeFn rows_encode() {
     return fn;
 }
 
-// activation [ni][h][w][Mp][C] bf16, boxes of (64, Mp, box_x, 1, 1), zeros outside
-bool rows_map_act(CUtensorMap *m, const void *ptr, int ni, int h, int w, int Mp, int C, int box_x) {
+// activation [ni][h][w][Mp][C] bf16, boxes of (64, Mp, box_x, box_y, 1), zeros outside
+bool rows_map_act(CUtensorMap *m, const void *ptr, int ni, int h, int w, int Mp, int C, int box_x, int box_y = 1) {
     RowsEncodeFn enc = rows_encode();
     if (!enc || box_x > 256) return false;
     cuuint64_t dims[5] = {(cuuint64_t)C, (cuuint64_t)Mp, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)ni};
     cuuint64_t strides[4] = {(cuuint64_t)C * 2, (cuuint64_t)Mp * C * 2, (cuuint64_t)w * Mp * C * 2,
                              (cuuint64_t)h * w * Mp * C * 2};
-    cuuint32_t box[5] = {64, (cuuint32_t)Mp, (cuuint32_t)box_x, 1, 1};
+    cuuint32_t box[5] = {64, (cuuint32_t)Mp, (cuuint32_t)box_x, (cuuint32_t)box_y, 1};
     cuuint32_t es[5] = {1, 1, 1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(ptr), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1247,6 +1483,72 @@ cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifC
         return cudaErrorInvalidValue;
     if (t.NT == 2) return rows_launch<64, 2, false>(mA, mB, a, p, st);
     return rows_launch<64, 1, false>(mA, mB, a, p, st);
+}
+
+// 3x3 layers at stride 1 with 64 output channels (1.1 to 1.4 times faster than a
+// box per tap, 0.97 on 3000 positions), and wider ones with 64 grid steps (128
+// -> 128 at 14 x 14: 1.37; 256 -> 256 at 7 x 7: 1.09). Wider ones with 32 grid
+// steps stay with a box per tap: a K step is then one position of 32, half of
+// whose MMA block (2, kw) is not used (1.07 at 64 input channels, 0.68 to 0.99
+// at 128 and more).
+bool conv_dw_cols_supported(const ConvGeom &g, int C_out, int Mp) {
+    return g.k == 3 && g.s == 1 && g.C % 64 == 0 &&
+           ((C_out == 64 && (Mp == 32 || Mp == 64)) || (C_out % 128 == 0 && Mp == 64));
+}
+
+cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *S,
+                                const __nv_bfloat16 *dW_hat, const float *count, float qcoef, float *g_W, int C_t,
+                                cudaStream_t st) {
+    if (!conv_dw_cols_supported(g, C_out, c.Mp)) return cudaErrorInvalidConfiguration;
+    DwColsPlan p{};
+    p.Ho = g.Ho;
+    p.Wo = g.Wo;
+    p.pad = g.p;
+    p.Mp = c.Mp;
+    p.ncb = g.C / 64;
+    const int BN = C_out == 64 ? 64 : 128;
+    p.n_col = C_out / BN;
+    p.rows = ni * g.Ho;
+    if (p.rows == 0) return cudaSuccess;
+    p.C_t = C_t;
+    p.g_W = g_W;
+    p.count = count;
+    p.qcoef = qcoef;
+    // ranges of rows: the fewest rounds of tiles on the SMs x (rows + the cost
+    // of a tile's epilogue, about two rows of 28 positions)
+    const int per = p.ncb * (BN == 64 ? 1 : 2) * p.n_col, sms = rows_num_sms();
+    const double tail = 56.0 / g.Wo;
+    double best = -1.0;
+    for (int n = 1; n <= p.rows && n <= 4 * sms; ++n) {
+        const int rp = (p.rows + n - 1) / n, ns = (p.rows + rp - 1) / rp;
+        const double cost = (double)(((long long)per * ns + sms - 1) / sms) * (rp + tail);
+        if (best < 0.0 || cost < best) {
+            best = cost;
+            p.rows_per = rp;
+            p.n_tiles = per * ns;
+        }
+    }
+    const int slot = ((BN == 64 ? 3 : 2) + BN / 64) * c.Mp * 128, extra = 1024 + (2 * DWC_MAX_RING + 2) * 8 + 8;
+    p.ring = (ROWS_SMEM_MAX - extra) / slot;
+    if (p.ring > DWC_MAX_RING) p.ring = DWC_MAX_RING;
+    if (p.ring < 4) return cudaErrorInvalidConfiguration;
+    CUtensorMap mS0, mS1, mD;
+    if (!rows_map_act(&mS0, S, ni, g.H, g.W, c.Mp, g.C, 1, BN == 64 ? 3 : 2) ||
+        !rows_map_act(&mS1, S, ni, g.H, g.W, c.Mp, g.C, 1, 1) ||
+        !rows_map_act(&mD, dW_hat, ni, g.Ho, g.Wo, c.Mp, C_out, 1, 1))
+        return cudaErrorInvalidValue;
+    const int smem = p.ring * slot + extra;
+    const int grid = p.n_tiles < sms ? p.n_tiles : sms;
+    if (BN == 64) {
+        cudaError_t e = cudaFuncSetAttribute(k_conv_dw_cols<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        k_conv_dw_cols<64><<<grid, DWC_THREADS, smem, st>>>(mS0, mS1, mD, p);
+    } else {
+        cudaError_t e = cudaFuncSetAttribute(k_conv_dw_cols<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        k_conv_dw_cols<128><<<grid, DWC_THREADS, smem, st>>>(mS0, mS1, mD, p);
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace dstd

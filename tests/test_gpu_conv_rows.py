@@ -1,4 +1,4 @@
-"""The conv contractions that take each source row once (the default path) against the one-row-at-a-time kernels
+"""The conv contractions that take each source row (dW: each column) once (the default path) against the one-row-at-a-time kernels
 (operand policy 2, whose results the conv parity tests hold to the oracle).
 
 Forward: the same products in the same order per output, so spike times and saved state are equal bit for bit.
@@ -100,6 +100,18 @@ def test_rows_match_one_row_at_a_time(case):
     assert torch.isfinite(a[0]).any()
     assert rel(a[2], b[2]) <= 1e-5
     assert rel(a[3], b[3]) <= 2e-5
+    assert rel(a[4], b[4]) <= 2e-5
+
+
+@pytest.mark.parametrize("case", [(3, 14, 14, 128, 128, 3, 1, 1, 64, (1.0, 0.25)), (2, 7, 9, 64, 256, 3, 1, 1, 50, (0.5, 0.25)),
+                                  (1, 1, 1, 64, 64, 3, 1, 1, 32, (INF, INF)), (5, 4, 3, 192, 64, 3, 1, 1, 20, (INF, INF)),
+                                  (2, 6, 5, 5, 64, 3, 1, 0, 64, (0.5, 0.25)), (700, 3, 3, 64, 128, 3, 1, 2, 40, (0.4, 0.2))],
+                         ids=lambda c: "-".join(str(x) for x in c[:9]))
+def test_weight_gradient_by_columns(case):
+    """dW of 3x3 layers at stride 1: both tile widths, several channel blocks and column tiles, padded channels, rows
+    split over few and many CTAs, a single position."""
+    a, b = run(*case, policy=0), run(*case, policy=2)
+    assert torch.equal(a[0], b[0]) and (b[4] != 0).any()
     assert rel(a[4], b[4]) <= 2e-5
 
 
