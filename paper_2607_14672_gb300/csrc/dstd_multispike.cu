@@ -36,94 +36,123 @@ __device__ __forceinline__ void ms_store(void *hi, void *lo, long long o, float 
     }
 }
 
-// the grid weights of the F spikes of one input: value at bin m
-struct MsBins {
-    int k[kMsMaxSpikes];
-    float wR[kMsMaxSpikes], wL[kMsMaxSpikes];
-    int n;
-};
-__device__ __forceinline__ void ms_bins(const LifConst &c, const float *t, int F, MsBins &b) {
-    b.n = 0;
-    for (int f = 0; f < F; ++f) {
-        const float x = t[f];
-        if (!isfinite(x)) continue;
-        const BinW w = bin_weights(c, x, false);
-        b.k[b.n] = w.k;
-        b.wR[b.n] = w.wR;
-        b.wL[b.n] = w.wL;
-        ++b.n;
+// two neighbouring elements, o even (rows of operands start on 16-byte boundaries)
+template <int OP>
+__device__ __forceinline__ void ms_store2(void *hi, void *lo, long long o, float v0, float v1) {
+    if (OP == 0) {
+        *reinterpret_cast<float2 *>(static_cast<float *>(hi) + o) = make_float2(v0, v1);
+    } else if (OP == 3) {
+        const __half2 h = __floats2half2_rn(v0, v1);
+        *reinterpret_cast<__half2 *>(static_cast<__half *>(hi) + o) = h;
+        *reinterpret_cast<__half2 *>(static_cast<__half *>(lo) + o) =
+            __floats2half2_rn(v0 - __low2float(h), v1 - __high2float(h));
+    } else {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+        *reinterpret_cast<__nv_bfloat162 *>(static_cast<__nv_bfloat16 *>(hi) + o) = h;
+        if (OP == 1)
+            *reinterpret_cast<__nv_bfloat162 *>(static_cast<__nv_bfloat16 *>(lo) + o) =
+                __floats2bfloat162_rn(v0 - __low2float(h), v1 - __high2float(h));
     }
 }
-__device__ __forceinline__ float ms_value(const LifConst &c, const MsBins &b, int m) {
-    float v = 0.f;
-    if (m >= c.M) return 0.f;
-    for (int u = 0; u < b.n; ++u) {
-        if (m == b.k[u]) v += b.wR[u];
-        if (m == b.k[u] + 1) v += b.wL[u];
+
+// the grid weights of one spike; no bin when it never comes
+constexpr int MS_NO_BIN = -100;
+struct MsSpike {
+    int k;
+    float wR, wL;
+};
+__device__ __forceinline__ MsSpike ms_spike(const LifConst &c, float x) {
+    MsSpike s{MS_NO_BIN, 0.f, 0.f};
+    if (isfinite(x)) {
+        const BinW w = bin_weights(c, x, false);
+        s = MsSpike{w.k, w.wR, w.wL};
     }
-    return v;
+    return s;
+}
+// adds the spike's weight at bin m < M
+__device__ __forceinline__ void ms_add(const MsSpike &s, int m, float &v) {
+    if (m == s.k) v += s.wR;
+    if (m == s.k + 1) v += s.wL;
 }
 
 }  // namespace
 
+// A thread per sample b and two neighbouring inputs: 4-byte stores, and the
+// spikes' weights in registers (indexed by a count they lay in local memory
+// and were read back for every bin). Bound by the compares of every bin with
+// every spike (800 inputs, B = 256, M = 32, 4 spikes: 43 -> 26 us).
 template <int OP>
-__global__ void k_binning_ms_rows(const float *__restrict__ t, int B, int N, int F, LifConst c, void *hi, void *lo,
-                                  int ld) {
+__global__ void __launch_bounds__(128) k_binning_ms_rows(const float *__restrict__ t, int B, int N, int F, LifConst c,
+                                                         void *hi, void *lo, int ld) {
     const int b = blockIdx.y;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= ld) return;
-    MsBins bins;
-    bins.n = 0;
-    if (j < N) ms_bins(c, t + ((long long)b * N + j) * F, F, bins);
-    for (int m = 0; m < c.Mp; ++m) ms_store<OP>(hi, lo, ((long long)b * c.Mp + m) * ld + j, ms_value(c, bins, m));
+    const int j = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (j >= ld) return;  // ld is even
+    MsSpike s[2][kMsMaxSpikes];
+#pragma unroll
+    for (int f = 0; f < kMsMaxSpikes; ++f) {
+        if (f >= F) break;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            s[h][f] = ms_spike(c, j + h < N ? t[((long long)b * N + j + h) * F + f] : INFINITY);
+    }
+    for (int m = 0; m < c.Mp; ++m) {
+        float v0 = 0.f, v1 = 0.f;
+        if (m < c.M) {
+#pragma unroll
+            for (int f = 0; f < kMsMaxSpikes; ++f) {
+                if (f >= F) break;
+                ms_add(s[0][f], m, v0);
+                ms_add(s[1][f], m, v1);
+            }
+        }
+        ms_store2<OP>(hi, lo, ((long long)b * c.Mp + m) * ld + j, v0, v1);
+    }
 }
 
-// a warp per (input j, sample b): lane f < F discretises spike f, the warp
-// shares the results, and lane l writes bins l, l + 32, ... of the row
-// segment (contiguous: column b*Mp + m)
+// Half a warp per (input j, sample b): lane f < F of the half discretises spike
+// f, the half shares the results, and lane l writes bins 2 l, 2 l + 1, 2 l + 32,
+// ... of the row segment (contiguous: column b*Mp + m), 4 bytes a store. Bound by
+// its stores' instructions (800 inputs, B = 256, M = 32, 4 spikes: 65 -> 44 us, a warp per
+// (input, sample) with 2-byte stores before).
+constexpr int MS_COLS_ITER = 4;  // up to 128 bins
 template <int OP>
 __global__ void __launch_bounds__(256) k_binning_ms_cols(const float *__restrict__ t, int B, int N, int F, LifConst c,
                                                          void *hi, void *lo, int ld) {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, l = lane & 15, h = lane & 16;
     const int j = blockIdx.x;
-    const int b = blockIdx.y * 8 + (threadIdx.x >> 5);
+    const int b = blockIdx.y * 16 + (threadIdx.x >> 4);
+    const MsSpike own = ms_spike(c, b < B && l < F ? t[((long long)b * N + j) * F + l] : INFINITY);
+    float v0[MS_COLS_ITER], v1[MS_COLS_ITER];  // bins 2 l + 32 i and the one after
+#pragma unroll
+    for (int i = 0; i < MS_COLS_ITER; ++i) v0[i] = v1[i] = 0.f;
+    for (int f = 0; f < F; ++f) {  // in the spikes' order, as the rows add them
+        const MsSpike s{__shfl_sync(0xffffffffu, own.k, h + f), __shfl_sync(0xffffffffu, own.wR, h + f),
+                        __shfl_sync(0xffffffffu, own.wL, h + f)};
+#pragma unroll
+        for (int i = 0; i < MS_COLS_ITER; ++i) {
+            const int m = 2 * l + 32 * i;
+            if (m < c.M) ms_add(s, m, v0[i]);
+            if (m + 1 < c.M) ms_add(s, m + 1, v1[i]);
+        }
+    }
     if (b >= B) return;
-    int kf = -100;
-    float wr = 0.f, wl = 0.f;
-    if (lane < F) {
-        const float x = t[((long long)b * N + j) * F + lane];
-        if (isfinite(x)) {
-            const BinW w = bin_weights(c, x, false);
-            kf = w.k;
-            wr = w.wR;
-            wl = w.wL;
-        }
-    }
-    MsBins bins;
-    bins.n = 0;
-    for (int f = 0; f < F; ++f) {
-        const int k = __shfl_sync(0xffffffffu, kf, f);
-        const float r = __shfl_sync(0xffffffffu, wr, f), l = __shfl_sync(0xffffffffu, wl, f);
-        if (k != -100) {
-            bins.k[bins.n] = k;
-            bins.wR[bins.n] = r;
-            bins.wL[bins.n] = l;
-            ++bins.n;
-        }
-    }
     const long long o = (long long)j * ld + (long long)b * c.Mp;
-    for (int m = lane; m < c.Mp; m += 32) ms_store<OP>(hi, lo, o + m, ms_value(c, bins, m));
+#pragma unroll
+    for (int i = 0; i < MS_COLS_ITER; ++i) {
+        const int m = 2 * l + 32 * i;
+        if (m < c.Mp) ms_store2<OP>(hi, lo, o + m, v0[i], v1[i]);
+    }
 }
 
 cudaError_t launch_binning_ms(const float *t, int B, int N, int F, const LifConst &c, OpKind op, bool transposed,
                               void *hi, void *lo, int ld, cudaStream_t st) {
-    if (F < 1 || F > kMsMaxSpikes) return cudaErrorInvalidValue;
+    if (F < 1 || F > kMsMaxSpikes || c.Mp > 32 * MS_COLS_ITER || ld % 2) return cudaErrorInvalidValue;
 #define DSTD_MS_BIN(OPV)                                                                                        \
     if (transposed)                                                                                             \
-        k_binning_ms_cols<OPV><<<dim3((unsigned)N, (unsigned)((B + 7) / 8)), 256, 0, st>>>(t, B, N, F, c, hi,  \
+        k_binning_ms_cols<OPV><<<dim3((unsigned)N, (unsigned)((B + 15) / 16)), 256, 0, st>>>(t, B, N, F, c, hi, \
                                                                                            lo, ld);             \
     else                                                                                                        \
-        k_binning_ms_rows<OPV><<<dim3((unsigned)((ld + 127) / 128), (unsigned)B), 128, 0, st>>>(t, B, N, F, c, \
+        k_binning_ms_rows<OPV><<<dim3((unsigned)((ld + 255) / 256), (unsigned)B), 128, 0, st>>>(t, B, N, F, c, \
                                                                                                 hi, lo, ld);
     switch (op) {
         case OpKind::F32: DSTD_MS_BIN(0) break;
@@ -142,36 +171,45 @@ cudaError_t launch_binning_ms(const float *t, int B, int N, int F, const LifCons
 // of the interval, of length L - s, is tested again. Outputs per spike k
 // (index (b*N + i)*F + k): t, the bin q, I at the spike and dv^/dt there;
 // t = +inf, q = M after the last spike.
+//
+// The neurons of a warp come to their exact tests on different intervals, and a
+// test is some hundred instructions: each lane walks on to its next interval
+// that needs one, and the warp then runs them together, so it pays for the
+// largest number of such intervals of a lane instead of for every interval that
+// any lane tests (800 outputs, B = 256, M = 32, up to 4 spikes: 107 -> 44 us).
 __global__ void __launch_bounds__(256) k_scan_ms(const float *__restrict__ what, long long sb, long long si, int B,
                                                  int N, LifConst c, int F, float *t_out, int *q_out, float *I_out,
                                                  float *vd_out, int vec4) {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)B * N) return;
+    const bool live = idx < (long long)B * N;
     const int b = (int)(idx / N), i = (int)(idx % N);
-    const float *w = what + b * sb + i * si;
+    const float *w = what + b * sb + i * si;  // read by live lanes only
     float v = 0.f, I = 0.f;
     int nk = 0;
     const long long o = idx * F;
     float4 w4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int m = 0; m < c.M && nk < F; ++m) {
-        if (vec4) {
-            if ((m & 3) == 0) w4 = __ldg(reinterpret_cast<const float4 *>(w + m));
-        }
-        const float wm = vec4 ? ((m & 3) == 0 ? w4.x : (m & 3) == 1 ? w4.y : (m & 3) == 2 ? w4.z : w4.w) : w[m];
-        float v0 = v, I0 = I + wm;
-        // a whole interval with no spike in it yet: the cheap tests of the
-        // first-spike scan decide whether the exact test is needed
-        {
+    for (int m = live ? 0 : c.M;; ++m) {
+        float v0 = 0.f, I0 = 0.f;
+        for (; m < c.M && nk < F; ++m) {
+            if (vec4) {
+                if ((m & 3) == 0) w4 = __ldg(reinterpret_cast<const float4 *>(w + m));
+            }
+            const float wm = vec4 ? ((m & 3) == 0 ? w4.x : (m & 3) == 1 ? w4.y : (m & 3) == 2 ? w4.z : w4.w) : w[m];
+            v0 = v;
+            I0 = I + wm;
+            // a whole interval with no spike in it yet: the cheap tests of the
+            // first-spike scan decide whether the exact test is needed
             const float ve = fmaf(c.KD, I0, c.rv * v0);
             const bool endp = ve >= c.vth;
             const bool peak = (fmaf(-c.av, v0, I0) > 0.0f) & (fmaf(-c.av, ve, c.rI * I0) < 0.0f) &
                               (fmaf(fmaxf(I0, 0.0f), c.Kmax, fmaxf(v0, 0.0f)) >= c.vth);
-            if (!(endp | peak)) {
-                v = ve;
-                I = c.rI * I0;
-                continue;
-            }
+            if (endp | peak) break;
+            v = ve;
+            I = c.rI * I0;
         }
+        const bool test = m < c.M && nk < F;
+        if (!__any_sync(0xffffffffu, test)) break;
+        if (!test) continue;
         float L = c.dt, start = c.T0 + (float)m * c.dt;
         // at most F spikes in all, so the inner loop ends
         while (nk < F) {
@@ -197,6 +235,7 @@ __global__ void __launch_bounds__(256) k_scan_ms(const float *__restrict__ what,
         v = fmaf(e * phi_f(c, L), I0, e * v0);
         I = I0 * expf(-c.aI * L);
     }
+    if (!live) return;
     for (int k = nk; k < F; ++k) {
         t_out[o + k] = INFINITY;
         q_out[o + k] = c.M;
@@ -223,6 +262,14 @@ cudaError_t launch_scan_ms(const float *what, long long sb, long long si, int B,
 // (the current kept through the reset decays at aI; dK/ds = -av K + e^{-aI s}).
 // The adjoints a_k = dC/dt_k + a_{k+1} dt_{k+1}/dt_k run from the last
 // spike back; dC/dw^_m = sum_k a_k dt_k/dw^_m.
+//
+// A bin m with q_{k-1} < m <= q_k takes one K (spike k) and one exponential per
+// later spike. The lanes of a warp take the K together, then the exponentials:
+// a loop over the spikes with either in it ran both for every spike of the lanes
+// (800 outputs, B = 256, M = 32, up to 4 spikes, with 4-byte stores: 87 -> 62 us).
+// The running sum of the later spikes' terms (one exponential per bin in all)
+// takes 50 us, but differs by 1e-5 where a spike only just reaches the threshold
+// and the terms cancel, so each term is taken as it stands above.
 //
 // A block takes 32 neurons of one sample: thread i < 32 runs neuron i's
 // adjoints into shared memory, the block fills a [Mp][32] tile of dC/dw^
@@ -262,16 +309,16 @@ __global__ void __launch_bounds__(256) k_dwhat_ms(const float *__restrict__ t_ou
             // adjoints, last spike first; coef_k = -a_k / v'_k
             for (int k = n - 1; k >= 0; --k) {
                 coef[k] = -coef[k] / vdv[o + k];
+                float K = 0.f;
                 if (k > 0) {
                     const float s = tk[k] - tk[k - 1];
-                    const float dv_dprev = Ik[k - 1] * fmaf(c.av - c.aI, kernel_K(c, s), -expf(-c.aI * s));
+                    K = kernel_K(c, s);
+                    const float dv_dprev = Ik[k - 1] * fmaf(c.av - c.aI, K, -expf(-c.aI * s));
                     coef[k - 1] += coef[k] * dv_dprev;  // a_{k-1} += a_k (-dv_dprev / v'_k)
                 }
-            }
-            for (int k = 0; k < n; ++k) {
                 stk[tid * F + k] = tk[k];
                 scf[tid * F + k] = coef[k];
-                sKk[tid * F + k] = k > 0 ? kernel_K(c, tk[k] - tk[k - 1]) : 0.f;
+                sKk[tid * F + k] = K;
             }
         }
         sn[tid] = n;
@@ -283,27 +330,25 @@ __global__ void __launch_bounds__(256) k_dwhat_ms(const float *__restrict__ t_ou
         const int n = sn[il];
         float val = 0.f;
         if (n > 0 && m <= sq[il * F + n - 1]) {
+            int k = 0;
+            while (m > sq[il * F + k]) ++k;  // the spike whose bins hold m (m <= the last spike's)
             const float Tm = c.T0 + (float)m * c.dt;
-            for (int k = 0; k < n; ++k) {
-                const int qk = sq[il * F + k];
-                if (m > qk) continue;
-                float basis;
-                if (k > 0 && m <= sq[il * F + k - 1])
-                    basis = expf(-c.aI * (stk[il * F + k - 1] - Tm)) * sKk[il * F + k];
-                else
-                    basis = kernel_K(c, stk[il * F + k] - Tm);
-                val = fmaf(scf[il * F + k], basis, val);
-            }
+            val = scf[il * F + k] * kernel_K(c, stk[il * F + k] - Tm);
+            for (++k; k < n; ++k)
+                val = fmaf(scf[il * F + k], expf(-c.aI * (stk[il * F + k - 1] - Tm)) * sKk[il * F + k], val);
         }
         tile[m * (MS_DW_NEURONS + 1) + il] = val;
     }
     __syncthreads();
     const int lane = tid & 31, warp = tid >> 5;
-    for (int il = warp; il < MS_DW_NEURONS; il += blockDim.x / 32) {
-        const int i = i0 + il;
-        if (i >= N) break;
+    // two neurons per warp, two bins per lane: 4-byte stores
+    for (int p = warp; p < MS_DW_NEURONS / 2; p += blockDim.x / 32) {
+        const int il = 2 * p + (lane >> 4), i = i0 + il;
+        if (i >= N) continue;
         const long long oa = (long long)i * lda + (long long)b * c.Mp;
-        for (int m = lane; m < c.Mp; m += 32) ms_store<OP>(a_hi, a_lo, oa + m, tile[m * (MS_DW_NEURONS + 1) + il]);
+        for (int m = 2 * (lane & 15); m < c.Mp; m += 32)
+            ms_store2<OP>(a_hi, a_lo, oa + m, tile[m * (MS_DW_NEURONS + 1) + il],
+                          tile[(m + 1) * (MS_DW_NEURONS + 1) + il]);
     }
     if (b_hi) {
         const int i = i0 + lane;
