@@ -187,7 +187,7 @@ int dstd_dense_bwd(const float *t_in, const float *W, const float *t_out, const 
  * compact support of Eq. DSTD_kernel); from those records the binned input
  * is either written out once per chunk ([images, H, W, Mp, C_in], no im2col
  * expansion) and read by the forward and dW through TMA boxes shifted per
- * filter tap, or generated tile by tap in shared memory
+ * filter tap, or generated in shared memory
  * (dstd_conv_set_operand_policy); dS is the transposed
  * convolution of dw^ (TMA boxes shifted per tap, only the taps on the
  * stride grid) with the input-time gradient taken in its epilogue. Chunks
@@ -363,11 +363,13 @@ int dstd_conv_set_chunk_images(int max_images);
  * 8-byte records; 2 writes it out once per chunk, S [images, H, W, Mp, C_in]
  * in bf16 (the two nonzero grid weights of each input at grid steps k and
  * k + 1, zeros elsewhere), and the contractions read it through TMA boxes
- * shifted per filter tap; 0 (the default) chooses per layer: forward and dS
- * by source rows where that is faster (see dstd_conv_fwd), else S wherever
- * its writer takes the channel count (C_in <= 256, or a multiple of 256 up to
- * 1024) and generated elsewhere. All compute the same products. It changes the workspace size, so query again after setting
- * it. Returns the previous value (a policy outside 0..2 only reads it).
+ * shifted per filter tap; 0 (the default) chooses per layer: where they are
+ * faster, kernels that take each source row or column once (the forward of
+ * large 64 -> 64 layers at stride 1, dS with 64 input channels, dW of 3x3
+ * layers at stride 1 with 64 output channels, or a multiple of 128 and
+ * 32 < M <= 64), else S wherever its writer takes the channel count (C_in <= 256, or a
+ * multiple of 256 up to 1024) and generated elsewhere. All compute the same
+ * products. It changes the workspace size, so query again after setting it. Returns the previous value (a policy outside 0..2 only reads it).
  * Process-wide; set it between calls. */
 int dstd_conv_set_operand_policy(int policy);
 

@@ -817,17 +817,20 @@ int conv_bwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
             else
                 TRY(cu(launch_conv_ds_gemm(gp, ni, C_out, c, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off, g.C, st)));
         }
+        const bool dw_cols = ws.S && g_conv_operand_policy == 0 && conv_dw_cols_supported(gp, C_out, Mp);
+        const bool dw_rec = dw_cols && conv_dw_cols_records(C_out);  // records in S's place, which is larger
+        uint2 *const rec = dw_rec ? reinterpret_cast<uint2 *>(ws.S) : ws.rec;
         {
             Timed tm(KK_BIN_T, st);
-            if (ws.S)
+            if (ws.S && !dw_rec)
                 TRY(cu(launch_bin_S(t_in + in_off, (long long)ni * g.H * g.W, gp.C, g.C, c, ws.S, st)));
             else
-                TRY(cu(launch_bin_rec(t_in + in_off, (long long)ni * g.H * g.W * g.C, c, ws.rec, st)));
+                TRY(cu(launch_bin_rec(t_in + in_off, (long long)ni * g.H * g.W * g.C, c, rec, st)));
         }
         Timed tm(KK_GEMM_DW, st);
-        if (ws.S && g_conv_operand_policy == 0 && conv_dw_cols_supported(gp, C_out, Mp))
-            TRY(cu(launch_conv_dw_cols(gp, ni, C_out, c, ws.S, ws.dwh, last ? ws.count : nullptr, qcoef, g_W, g.C,
-                                       st)));
+        if (dw_cols)
+            TRY(cu(launch_conv_dw_cols(gp, ni, C_out, c, dw_rec ? rec : nullptr, ws.S, ws.dwh,
+                                       last ? ws.count : nullptr, qcoef, g_W, g.C, st)));
         else if (ws.S)
             TRY(cu(launch_conv_dw_tma(gp, ni, C_out, c, ws.S, ws.dwh, last ? ws.count : nullptr, qcoef, g_W, g.C,
                                       st)));

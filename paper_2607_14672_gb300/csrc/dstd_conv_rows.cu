@@ -27,7 +27,7 @@
 // or (filter column, channel block) as those take them for the same shape, so
 // both give the same w^.
 //
-// dW of 3x3 layers at stride 1 (k_conv_dw_cols) reads each column of the binned
+// dW of 3x3 layers at stride 1 (k_conv_dw_cols) takes each column of the binned
 // input once in the same spirit.
 //
 // Every mbarrier wait is bounded; an expired wait sets this unit's status
@@ -920,62 +920,82 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
 // dW of 3x3 layers at stride 1, walking the output rows position by position:
 //   dW[o, (kh, kw), c] = sum_{y, x, m} dw^[(y, x, m), o] S[(y + kh, x + kw, m), c]
 // A K step is one output position (Mp grid steps). Its nine taps read three
-// columns of S, two of which the step before has read: a ring of columns in
-// shared memory (the S boxes of the rows y - pad .. for one x, one copy each,
-// and the dw^ box of the position that the column completes) is filled once
-// per position where a box per tap and position was loaded before: 32 KB
-// instead of 88 KB per step (64 channels, Mp = 64), with three and more
-// columns in flight instead of one step.
+// columns of S, two of which the step before has taken: a ring of columns in
+// shared memory (the S boxes of the rows y - pad .. for one x, and the dw^ box
+// of the position that the column completes) is filled once per position where
+// a box per tap and position was loaded before: 32 KB instead of 88 KB per step
+// (64 channels, Mp = 64), with three and more columns in flight instead of one
+// step. With 64 output channels generator warps write the columns from 8 bytes
+// per input spike, so that the backward writes no S; with 128 the MMAs of a
+// column are too short for them (128 -> 128 at 14 x 14: 0.84 ms generated,
+// 0.58 ms from S) and S comes by TMA.
 // The filter rows of the layer's channel block form 128-row MMA blocks: the
 // taps (0, kw) and (1, kw) together (their boxes lie side by side), tap
 // (2, kw) alone (the other 64 rows of the block are not used); with 64 output
 // channels per tile all six blocks share a CTA, with 128 the first three and
 // the last three are tiles of their own (TMEM holds four accumulators of 128
 // columns). Split over output rows; fp32 atomics into g_W. Warps: 0 TMA, 1-4
-// MMA issue (block b by warp b mod 4), 5-12 epilogue. Bound by the MMAs' reads
-// of shared memory. Measured, a box per tap before and by columns (B = 256,
-// M = 64): 64 -> 64 at 28 x 28 1.29 -> 0.90 ms, 128 -> 128 at 14 x 14
-// 0.79 -> 0.57 ms.
+// MMA issue (block b by warp b mod 4), 5-12 epilogue, 13.. generators. Bound by
+// the MMAs' reads of shared memory. Measured, a box per tap before and by columns
+// (B = 256, M = 64): 64 -> 64 at 28 x 28 1.29 -> 0.92 ms
+// (and 0.27 ms of writing S -> 0.07 of records), 128 -> 128 at 14 x 14 0.79 -> 0.61.
 // ---------------------------------------------------------------------------
 constexpr int DWC_MAX_RING = 8;
 constexpr int DWC_MMA_WARPS = 4;
-constexpr int DWC_THREADS = (1 + DWC_MMA_WARPS + 8) * 32;
+template <int BN>
+struct DwCols {
+    static constexpr bool GEN = BN == 64;           // columns generated on chip, else S by TMA
+    static constexpr int BOXES = BN == 64 ? 3 : 2;  // source boxes of a slot
+    static constexpr int GW = GEN ? 2 * BOXES : 0;  // generator warps: two per box, a thread per channel
+    static constexpr int THREADS = (1 + DWC_MMA_WARPS + 8 + GW) * 32;
+    static constexpr int SLOT_BOXES = BOXES + BN / 64;
+    static constexpr int EXTRA = 1024 + (2 * DWC_MAX_RING + 2) * 8 + 8 + DWC_MAX_RING * GW * 32;  // beside the ring
+};
 
 struct DwColsPlan {
-    int Ho, Wo, pad, Mp, ncb, n_col;
+    int H, W, Ho, Wo, pad, M, Mp, ncb, n_col;
     int rows, rows_per, n_tiles, ring;
-    int C_t;              // the layer's input channels (below 64: padded to 64 in S)
+    const uint2 *rec;     // [ni H W][C_t] records of the input
+    int C_t;              // the layer's input channels (below 64: padded to 64)
     float *g_W;           // [C_out][9][C_t]
     const float *count;   // silent neurons per output channel, or null
     float qcoef;
 };
 
 template <int BN>
-__global__ void __launch_bounds__(DWC_THREADS, 1)
+__global__ void __launch_bounds__(DwCols<BN>::THREADS, 1)
     k_conv_dw_cols(const __grid_constant__ CUtensorMap mapS0, const __grid_constant__ CUtensorMap mapS1,
                    const __grid_constant__ CUtensorMap mapD, const __grid_constant__ DwColsPlan p) {
-    constexpr int NGRP = BN == 64 ? 1 : 2;
+    constexpr int NGRP = BN == 64 ? 1 : 2, NBOX = DwCols<BN>::BOXES, GW = DwCols<BN>::GW;
+    constexpr bool GEN = DwCols<BN>::GEN;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int box = p.Mp * 128;
-    const int slot_bytes = ((NGRP == 1 ? 3 : 2) + BN / 64) * box;  // (the second group's slots are one box smaller)
+    const int slot_bytes = DwCols<BN>::SLOT_BOXES * box;  // (the second group leaves one source box unused)
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + p.ring * slot_bytes);
     uint64_t *empty = full + DWC_MAX_RING;
     uint64_t *acc_full = empty + DWC_MAX_RING;
     uint64_t *acc_empty = acc_full + 1;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 1);
+    int8_t *kept = reinterpret_cast<int8_t *>(tmem_slot + 2);  // [ring][GW 32] grid steps in the boxes
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int per = p.ncb * NGRP * p.n_col;  // tiles of one range of rows
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < DWC_MAX_RING; ++s) {
-            tc::mbar_init(&full[s], 1);
+            tc::mbar_init(&full[s], 1 + GW);
             tc::mbar_init(&empty[s], DWC_MMA_WARPS);
         }
         tc::mbar_init(acc_full, DWC_MMA_WARPS);
         tc::mbar_init(acc_empty, 8);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (GEN) {  // zero boxes and no kept steps: the generators then write only nonzeros
+        for (int i = threadIdx.x; i < p.ring * slot_bytes / 16; i += blockDim.x)
+            reinterpret_cast<uint4 *>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = threadIdx.x; i < p.ring * GW * 32; i += blockDim.x) kept[i] = (int8_t)SILENT;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) tc::tmem_alloc(tmem_slot, 512);
     tc::tc_fence_before();
@@ -1004,7 +1024,7 @@ __global__ void __launch_bounds__(DWC_THREADS, 1)
         for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
             int r0, r1, cb, grp, ct;
             decode(t, r0, r1, cb, grp, ct);
-            const int nbox = NGRP == 1 ? 3 : 2 - grp, kh0 = NGRP == 1 ? 0 : 2 * grp;
+            const int nbox = GEN ? 0 : 2 - grp;  // source boxes of a column that come by TMA
             int b = r0 / p.Ho, y = r0 - b * p.Ho;
             for (int r = r0; r < r1 && ok; ++r) {
                 for (int cx = 0; cx < p.Wo + 2; ++cx, ++n) {
@@ -1015,12 +1035,13 @@ __global__ void __launch_bounds__(DWC_THREADS, 1)
                     // columns 0 and 1 complete no position
                     tc::mbar_expect_tx_if(lead, &full[s], (uint32_t)((nbox + (cx >= 2 ? BN / 64 : 0)) * box));
                     const uint32_t st = tc::smem_u32(smem + s * slot_bytes);
-                    tc::tma_load_5d_if(lead, st, grp == 0 ? &mapS0 : &mapS1, &full[s], cb * 64, 0, cx - p.pad,
-                                       y - p.pad + kh0, b);
+                    if (!GEN)
+                        tc::tma_load_5d_if(lead, st, grp == 0 ? &mapS0 : &mapS1, &full[s], cb * 64, 0, cx - p.pad,
+                                           y - p.pad + 2 * grp, b);
                     if (cx >= 2)
 #pragma unroll
                         for (int h = 0; h < BN / 64; ++h)
-                            tc::tma_load_5d_if(lead, st + (uint32_t)((nbox + h) * box), &mapD, &full[s],
+                            tc::tma_load_5d_if(lead, st + (uint32_t)((NBOX + h) * box), &mapD, &full[s],
                                                ct * BN + h * 64, 0, cx - 2, y, b);
                     if (++s == p.ring) {
                         s = 0;
@@ -1054,7 +1075,6 @@ __global__ void __launch_bounds__(DWC_THREADS, 1)
         for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x, ++j) {
             int r0, r1, cb, grp, ct;
             decode(t, r0, r1, cb, grp, ct);
-            const int nbox = NGRP == 1 ? 3 : 2 - grp;
             constexpr int NBLK = NGRP == 1 ? 6 : 3;
             if (j >= 1) {
                 if (!tc::mbar_wait_warp(acc_empty, (j - 1) & 1u)) {
@@ -1075,7 +1095,7 @@ __global__ void __launch_bounds__(DWC_THREADS, 1)
                         const uint32_t cols =
                             tc::uniform((uint32_t)(back(s, 2) | (back(s, 1) << 8) | (s << 16)));  // slots of kw = 0, 1, 2
                         if (lead) {
-                            const uint32_t blo = base + ((cols >> 16) * (uint32_t)slot_bytes + (uint32_t)(nbox * box)) / 16u;
+                            const uint32_t blo = base + ((cols >> 16) * (uint32_t)slot_bytes + (uint32_t)(NBOX * box)) / 16u;
                             for (int bk = mw; bk < NBLK; bk += DWC_MMA_WARPS) {
                                 const int kw = bk < 3 ? bk : bk - 3, bx = bk < 3 ? 0 : 2;
                                 const uint32_t alo =
@@ -1103,6 +1123,77 @@ __global__ void __launch_bounds__(DWC_THREADS, 1)
             if (ok) tc::mma_commit_if(lead, acc_full);
         }
         if (!ok && lead) rows_set_status(STATUS_TIMEOUT);
+        __syncwarp();
+    } else if (GEN && warp > DWC_MMA_WARPS + 8) {
+        // Generators: warps 2 h and 2 h + 1 write box h of every column, a
+        // thread one channel; its record is loaded one column ahead.
+        const int gi = threadIdx.x - (1 + DWC_MMA_WARPS + 8) * 32, h = gi >> 6, c = gi & 63;
+        struct Col {
+            int t, r, r1, cx, b, y, cb;
+        };
+        auto open = [&](Col &q) {
+            int r0, grp, ct;
+            decode(q.t, r0, q.r1, q.cb, grp, ct);
+            q.r = r0;
+            q.cx = 0;
+            q.b = r0 / p.Ho;
+            q.y = r0 - q.b * p.Ho;
+        };
+        auto step = [&](Col &q) {
+            if (++q.cx < p.Wo + 2) return;
+            q.cx = 0;
+            if (++q.y == p.Ho) {
+                q.y = 0;
+                ++q.b;
+            }
+            if (++q.r == q.r1) {
+                q.t += gridDim.x;
+                if (q.t < p.n_tiles) open(q);
+            }
+        };
+        auto load = [&](const Col &q) {
+            const int y = q.y - p.pad + h, x = q.cx - p.pad, ch = q.cb * 64 + c;
+            if (q.t >= p.n_tiles || y < 0 || y >= p.H || x < 0 || x >= p.W || ch >= p.C_t)
+                return make_uint2((uint32_t)SILENT, 0u);
+            return __ldg(p.rec + (((long long)q.b * p.H + y) * p.W + x) * p.C_t + ch);
+        };
+        Col q, nx;
+        nx.t = blockIdx.x;
+        if (nx.t < p.n_tiles) open(nx);
+        q = nx;
+        uint2 tn = load(nx);
+        int s = 0;
+        uint32_t ph = 0;
+        for (; q.t < p.n_tiles; step(q)) {
+            const uint2 cur = tn;
+            step(nx);
+            tn = load(nx);
+            int got = 1;
+            if (lane == 0) got = tc::mbar_wait_spin(&empty[s], ph ^ 1u) ? 1 : 0;
+            if (!__shfl_sync(0xffffffffu, got, 0)) {
+                if (lane == 0) rows_set_status(STATUS_TIMEOUT);
+                break;
+            }
+            const uint32_t bx = tc::smem_u32(smem + s * slot_bytes + h * box);
+            int8_t *kp = kept + s * GW * 32 + gi;
+            const int kk = (int)cur.x, old = *kp;
+            if (old != SILENT) {
+                if (old >= 0) rows_sts_u16(bx + rows_sw128(old, c), 0);
+                if (old + 1 < p.M) rows_sts_u16(bx + rows_sw128(old + 1, c), 0);
+            }
+            if (kk != SILENT) {
+                if (kk >= 0) rows_sts_u16(bx + rows_sw128(kk, c), (uint16_t)(cur.y & 0xffffu));
+                if (kk + 1 < p.M) rows_sts_u16(bx + rows_sw128(kk + 1, c), (uint16_t)(cur.y >> 16));
+            }
+            if (kk != old) *kp = (int8_t)kk;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&full[s]);
+            if (++s == p.ring) {
+                s = 0;
+                ph ^= 1u;
+            }
+        }
         __syncwarp();
     } else {
         const int quarter = warp & 3, half = (warp - 1 - DWC_MMA_WARPS) >> 2;
@@ -1491,16 +1582,22 @@ cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifC
 // steps stay with a box per tap: a K step is then one position of 32, half of
 // whose MMA block (2, kw) is not used (1.07 at 64 input channels, 0.68 to 0.99
 // at 128 and more).
+bool conv_dw_cols_records(int C_out) { return C_out == 64; }
+
 bool conv_dw_cols_supported(const ConvGeom &g, int C_out, int Mp) {
     return g.k == 3 && g.s == 1 && g.C % 64 == 0 &&
            ((C_out == 64 && (Mp == 32 || Mp == 64)) || (C_out % 128 == 0 && Mp == 64));
 }
 
-cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *S,
-                                const __nv_bfloat16 *dW_hat, const float *count, float qcoef, float *g_W, int C_t,
+cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const uint2 *rec,
+                                const __nv_bfloat16 *S, const __nv_bfloat16 *dW_hat, const float *count, float qcoef, float *g_W, int C_t,
                                 cudaStream_t st) {
     if (!conv_dw_cols_supported(g, C_out, c.Mp)) return cudaErrorInvalidConfiguration;
     DwColsPlan p{};
+    p.H = g.H;
+    p.W = g.W;
+    p.M = c.M;
+    p.rec = rec;
     p.Ho = g.Ho;
     p.Wo = g.Wo;
     p.pad = g.p;
@@ -1515,11 +1612,18 @@ cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifC
     p.count = count;
     p.qcoef = qcoef;
     // ranges of rows: the fewest rounds of tiles on the SMs x (rows + the cost
-    // of a tile's epilogue, about two rows of 28 positions)
+    // of a tile's epilogue, about two rows of 28 positions), but at least as
+    // many as splits in k_conv_dw_tma, with 128 columns half as many again: the
+    // tensor core cuts its sums off, so the error of a range grows with its
+    // length. With one round of tiles dW of 64 -> 64 at 28 x 28 was 24e-6 off and
+    // of 128 -> 128 at 14 x 14 8e-6, against 16e-6 and 2e-6 of that kernel.
     const int per = p.ncb * (BN == 64 ? 1 : 2) * p.n_col, sms = rows_num_sms();
+    const int G = BN == 64 ? 5 : 3, row_tiles = (9 * p.ncb + 1) / 2;
+    int least = (BN == 64 ? 2 : 3) * sms / ((row_tiles + G - 1) / G * p.n_col);
+    if (least > p.rows) least = p.rows;
     const double tail = 56.0 / g.Wo;
     double best = -1.0;
-    for (int n = 1; n <= p.rows && n <= 4 * sms; ++n) {
+    for (int n = least < 1 ? 1 : least; n <= p.rows && (n <= least || n <= 4 * sms); ++n) {
         const int rp = (p.rows + n - 1) / n, ns = (p.rows + rp - 1) / rp;
         const double cost = (double)(((long long)per * ns + sms - 1) / sms) * (rp + tail);
         if (best < 0.0 || cost < best) {
@@ -1528,25 +1632,26 @@ cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifC
             p.n_tiles = per * ns;
         }
     }
-    const int slot = ((BN == 64 ? 3 : 2) + BN / 64) * c.Mp * 128, extra = 1024 + (2 * DWC_MAX_RING + 2) * 8 + 8;
+    const int slot = (BN == 64 ? DwCols<64>::SLOT_BOXES : DwCols<128>::SLOT_BOXES) * c.Mp * 128;
+    const int extra = BN == 64 ? DwCols<64>::EXTRA : DwCols<128>::EXTRA;
     p.ring = (ROWS_SMEM_MAX - extra) / slot;
     if (p.ring > DWC_MAX_RING) p.ring = DWC_MAX_RING;
     if (p.ring < 4) return cudaErrorInvalidConfiguration;
-    CUtensorMap mS0, mS1, mD;
-    if (!rows_map_act(&mS0, S, ni, g.H, g.W, c.Mp, g.C, 1, BN == 64 ? 3 : 2) ||
-        !rows_map_act(&mS1, S, ni, g.H, g.W, c.Mp, g.C, 1, 1) ||
-        !rows_map_act(&mD, dW_hat, ni, g.Ho, g.Wo, c.Mp, C_out, 1, 1))
+    CUtensorMap mS0{}, mS1{}, mD;
+    if (!rec && (!rows_map_act(&mS0, S, ni, g.H, g.W, c.Mp, g.C, 1, 2) ||
+                 !rows_map_act(&mS1, S, ni, g.H, g.W, c.Mp, g.C, 1)))
         return cudaErrorInvalidValue;
+    if (!rows_map_act(&mD, dW_hat, ni, g.Ho, g.Wo, c.Mp, C_out, 1)) return cudaErrorInvalidValue;
     const int smem = p.ring * slot + extra;
     const int grid = p.n_tiles < sms ? p.n_tiles : sms;
     if (BN == 64) {
         cudaError_t e = cudaFuncSetAttribute(k_conv_dw_cols<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        k_conv_dw_cols<64><<<grid, DWC_THREADS, smem, st>>>(mS0, mS1, mD, p);
+        k_conv_dw_cols<64><<<grid, DwCols<64>::THREADS, smem, st>>>(mS0, mS1, mD, p);
     } else {
         cudaError_t e = cudaFuncSetAttribute(k_conv_dw_cols<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        k_conv_dw_cols<128><<<grid, DWC_THREADS, smem, st>>>(mS0, mS1, mD, p);
+        k_conv_dw_cols<128><<<grid, DwCols<128>::THREADS, smem, st>>>(mS0, mS1, mD, p);
     }
     return cudaGetLastError();
 }

@@ -1612,8 +1612,8 @@ __global__ void __launch_bounds__(DW_THREADS, 1)
 // with the A tiles loaded instead of generated: per K step and row block
 // (tap, 64 channels) one box (64 channels, Mp grid steps) of S per output
 // position of the step, at the input position the tap reads (outside the
-// image: zeros), and BN / 64 boxes of dw^. Warps: 0 TMA (one lane), 1 MMA,
-// 2-9 epilogue (fp32 atomics into g_W, dead-neuron term on the first split).
+// image: zeros), and BN / 64 boxes of dw^. Warps: 0 TMA, 1-4 MMA, 5-12
+// epilogue (fp32 atomics into g_W, dead-neuron term on the first split).
 // ---------------------------------------------------------------------------
 constexpr int DWT_MAX_STAGES = 8;
 // The row tiles of a K step go round the issuing warps (each tile its own

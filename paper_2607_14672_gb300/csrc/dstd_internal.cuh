@@ -514,11 +514,13 @@ cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const Lif
 bool conv_rows_ds_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner);
 cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
                                 const __nv_bfloat16 *dW_hat, const __nv_bfloat16 *Wt, const float *t_in, float *g_t_in, int C_t, cudaStream_t st);
-// dW of 3x3 layers at stride 1, each column of S read once per channel block
-// (same file; arguments as launch_conv_dw_tma)
+// dW of 3x3 layers at stride 1, each column of S taken once per channel block
+// (same file; as launch_conv_dw_tma): generated from the records [ni H W][C_t]
+// where conv_dw_cols_records says so, else (rec null) read from S
 bool conv_dw_cols_supported(const ConvGeom &g, int C_out, int Mp);
-cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *S,
-                                const __nv_bfloat16 *dW_hat, const float *count, float qcoef, float *g_W, int C_t,
+bool conv_dw_cols_records(int C_out);
+cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const uint2 *rec,
+                                const __nv_bfloat16 *S, const __nv_bfloat16 *dW_hat, const float *count, float qcoef, float *g_W, int C_t,
                                 cudaStream_t st);
 cudaError_t conv_rows_status_read(unsigned int *out, int clear);
 // dW from S and dw^ (added into g_W as for launch_conv_dw_gen)
