@@ -711,7 +711,11 @@ def conv_step_units(n):
                     weights per input spike), with the dense tensor-core
                     flops of the binned formulation beside them;
       binning       read the input spike times (4 B), write the binned
-                    operand in the NHWC + grid-step layout (M x 2 B each);
+                    operand in the NHWC + grid-step layout (M x 2 B each),
+                    or, for layers whose contraction generates it on chip
+                    (the library's rules for the forward of large 64 -> 64
+                    layers and for dW of 3x3 layers with 64 outputs), an
+                    8-byte record;
       scan/solve    read w^ (positions x M_p x C_out x 4 B), write 16 B per neuron;
       dw^           read 20 B per neuron, write positions x M_p x C_out x 2 B;
       weight prep   read W (4 B), write its bf16 copy (forward and, where the
@@ -739,8 +743,11 @@ def conv_step_units(n):
             for kk in kinds:
                 add(algo_f, kk, f)
                 add(dense_f, kk, df)
-            add(algo_b, "binning", Pin * 4 + Pin * M * 2)
-            add(algo_b, "binning_T", Pin * 4 + Pin * M * 2)
+            on_chip = n.math == "bf16" and O == 64 and st == 1 and Mp in (32, 64)
+            rec_fwd = on_chip and C <= 64 and k > 1 and P >= 300 * 152
+            rec_bwd = on_chip and k == 3
+            add(algo_b, "binning", Pin * 4 + Pin * (8 if rec_fwd else M * 2))
+            add(algo_b, "binning_T", Pin * 4 + Pin * (8 if rec_bwd else M * 2))
             add(algo_b, "scan_solve", P * O * Mp * 4 + P * O * 16)
             add(algo_b, "dwhat", P * O * 20 + P * O * Mp * 2)
             add(algo_b, "prep_weights", (O * K * 6) * (2 if l > 0 else 1))
