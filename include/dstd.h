@@ -374,6 +374,22 @@ int dstd_conv_set_chunk_images(int max_images);
  * Process-wide; set it between calls. */
 int dstd_conv_set_operand_policy(int policy);
 
+/* The kernels that the calls of a conv layer take under the settings above:
+ * 0 for the im2col path, else DSTD_ROUTE_IMPLICIT and the bits of its chunks
+ * of the full size (a smaller last chunk may take others), or a DSTD_E_*
+ * code (negative) where the layer is refused. */
+enum {
+    DSTD_ROUTE_IMPLICIT = 1,    /* implicit GEMM: no im2col operand */
+    DSTD_ROUTE_FUSED_SCAN = 2,  /* the scan runs in the forward contraction: no w^ in memory */
+    DSTD_ROUTE_FWD_BINNED = 4,  /* the forward reads the binned input S, else 8-byte records */
+    DSTD_ROUTE_FWD_ROWS = 8,    /* each source row taken once */
+    DSTD_ROUTE_DS_ROWS = 16,    /* dS: each source row of dw^ taken once */
+    DSTD_ROUTE_DW_BINNED = 32,  /* dW reads the binned input S, else 8-byte records */
+    DSTD_ROUTE_DW_COLUMNS = 64  /* dW: each column of S taken once */
+};
+int dstd_conv_route(int B, int H, int W, int C_in, int C_out, int k, int stride, int pad, const dstd_params *p,
+                    dstd_math math);
+
 /* Kernel timing (tracing). While enabled, the library brackets every kernel
  * it launches with a CUDA event pair on the launching stream and files the
  * pair under the kernel's kind (dstd_kernel_kind_name). Kernels that

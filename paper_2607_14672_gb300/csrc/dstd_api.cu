@@ -713,6 +713,34 @@ bool conv_use_implicit(dstd_math math, const ConvGeom &g, int C_out, int Mp) {
     return math == DSTD_MATH_BF16 && conv_implicit_supported(g, C_out, Mp);
 }
 
+// The kernels that a chunk of ni images takes; dstd_conv_route reports them.
+struct ConvFwdRoute {
+    bool S;         // the contraction reads the binned input written out
+    bool rows;      // by source rows, from records (in S's place, which is larger)
+    bool cb_inner;  // order of its products (see conv_fwd_row_boxes)
+};
+static ConvFwdRoute conv_fwd_route(const ConvGeom &g, int ni, int C_out, int Mp) {
+    const ConvGeom gp = conv_padded(g);
+    ConvFwdRoute r{conv_fwd_tma(g, C_out), false, !conv_fwd_row_boxes(gp, C_out, Mp)};
+    r.rows = r.S && g_conv_operand_policy == 0 && conv_rows_fwd_supported(gp, ni, C_out, Mp, r.cb_inner);
+    if (r.rows) r.S = false;
+    return r;
+}
+struct ConvBwdRoute {
+    bool ds_rows, ds_cb_inner;  // dS by source rows, and the order of its products
+    bool dw_cols;               // dW by columns
+    bool dw_S;                  // dW reads the binned input written out, else records
+};
+static ConvBwdRoute conv_bwd_route(const ConvGeom &g, int ni, int C_out, int Mp) {
+    const ConvGeom gp = conv_padded(g);
+    ConvBwdRoute r{false, !conv_ds_row_boxes(gp, C_out, Mp), false, conv_dw_tma(g, C_out)};
+    if (g_conv_operand_policy != 0) return r;
+    r.ds_rows = conv_rows_ds_supported(gp, ni, C_out, Mp, r.ds_cb_inner);
+    r.dw_cols = r.dw_S && conv_dw_cols_supported(gp, C_out, Mp);
+    if (r.dw_cols && conv_dw_cols_records(C_out)) r.dw_S = false;
+    return r;
+}
+
 int conv_fwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int C_out, const dstd_params *p, int Mp,
                       float *t_out, void *saved, float *penalty, void *workspace, size_t ws_bytes, cudaStream_t st) {
     const ConvImplWs ws = conv_impl_layout(workspace, g, C_out, Mp, true);
@@ -736,33 +764,32 @@ int conv_fwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
                                        ws.rowsum, st)));
         }
     }
-    const bool cb_inner = !conv_fwd_row_boxes(gp, C_out, Mp);
     for (int img0 = 0; img0 < g.B; img0 += ws.imgs) {
         const int ni = (g.B - img0) < ws.imgs ? (g.B - img0) : ws.imgs;
+        const ConvFwdRoute rt = conv_fwd_route(g, ni, C_out, Mp);
         const long long in_off = (long long)img0 * g.H * g.W * g.C;
         const long long out_off = (long long)img0 * g.Ho * g.Wo * C_out;
         const long long P_out = (long long)ni * g.Ho * g.Wo;
-        if (g_conv_operand_policy == 0 && ws.S && conv_rows_fwd_supported(gp, ni, C_out, Mp, cb_inner)) {
-            // 8 bytes per input (in S's place, which is larger), then contraction and scan in one kernel
+        if (rt.rows) {  // 8 bytes per input, then contraction and scan in one kernel
             uint2 *rec = reinterpret_cast<uint2 *>(ws.S);
             {
                 Timed tm(KK_BIN, st);
                 TRY(cu(launch_bin_rec(t_in + in_off, (long long)ni * g.H * g.W * g.C, c, rec, st)));
             }
             Timed tm(KK_GEMM_FWD, st);
-            TRY(cu(launch_conv_rows_fwd(gp, ni, C_out, c, cb_inner, rec, g.C, ws.Wf, ws.rowsum,
+            TRY(cu(launch_conv_rows_fwd(gp, ni, C_out, c, rt.cb_inner, rec, g.C, ws.Wf, ws.rowsum,
                                         t_out + out_off, sv.q + out_off, sv.s + out_off, sv.vdot + out_off, penalty,
                                         st)));
             continue;
         }
         {
             Timed tm(KK_BIN, st);
-            if (ws.S)
+            if (rt.S)
                 TRY(cu(launch_bin_S(t_in + in_off, (long long)ni * g.H * g.W, gp.C, g.C, c, ws.S, st)));
             else
                 TRY(cu(launch_bin_rec(t_in + in_off, (long long)ni * g.H * g.W * g.C, c, ws.rec, st)));
         }
-        if (ws.S) {  // the scan runs in the contraction's epilogue
+        if (rt.S) {  // the scan runs in the contraction's epilogue
             Timed tm(KK_GEMM_FWD, st);
             TRY(cu(launch_conv_fwd_tma(gp, ni, C_out, c, ws.S, ws.Wf, ws.rowsum, t_out + out_off, sv.q + out_off,
                                        sv.s + out_off, sv.vdot + out_off, penalty, st)));
@@ -800,6 +827,7 @@ int conv_bwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
     for (int img0 = 0; img0 < g.B; img0 += ws.imgs) {
         const int ni = (g.B - img0) < ws.imgs ? (g.B - img0) : ws.imgs;
         const bool last = img0 + ni >= g.B;
+        const ConvBwdRoute rt = conv_bwd_route(g, ni, C_out, Mp);
         const long long in_off = (long long)img0 * g.H * g.W * g.C;
         const long long out_off = (long long)img0 * g.Ho * g.Wo * C_out;
         const long long P_out = (long long)ni * g.Ho * g.Wo;
@@ -810,28 +838,25 @@ int conv_bwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
         }
         if (g_t_in) {
             Timed tm(KK_GEMM_DS, st);
-            const bool cb_inner = !conv_ds_row_boxes(gp, C_out, Mp);
-            if (g_conv_operand_policy == 0 && conv_rows_ds_supported(gp, ni, C_out, Mp, cb_inner))
-                TRY(cu(launch_conv_rows_ds(gp, ni, C_out, c, cb_inner, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off,
+            if (rt.ds_rows)
+                TRY(cu(launch_conv_rows_ds(gp, ni, C_out, c, rt.ds_cb_inner, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off,
                                            g.C, st)));
             else
                 TRY(cu(launch_conv_ds_gemm(gp, ni, C_out, c, ws.dwh, ws.Wt, t_in + in_off, g_t_in + in_off, g.C, st)));
         }
-        const bool dw_cols = ws.S && g_conv_operand_policy == 0 && conv_dw_cols_supported(gp, C_out, Mp);
-        const bool dw_rec = dw_cols && conv_dw_cols_records(C_out);  // records in S's place, which is larger
-        uint2 *const rec = dw_rec ? reinterpret_cast<uint2 *>(ws.S) : ws.rec;
+        uint2 *const rec = ws.S ? reinterpret_cast<uint2 *>(ws.S) : ws.rec;  // in S's place, which is larger
         {
             Timed tm(KK_BIN_T, st);
-            if (ws.S && !dw_rec)
+            if (rt.dw_S)
                 TRY(cu(launch_bin_S(t_in + in_off, (long long)ni * g.H * g.W, gp.C, g.C, c, ws.S, st)));
             else
                 TRY(cu(launch_bin_rec(t_in + in_off, (long long)ni * g.H * g.W * g.C, c, rec, st)));
         }
         Timed tm(KK_GEMM_DW, st);
-        if (dw_cols)
-            TRY(cu(launch_conv_dw_cols(gp, ni, C_out, c, dw_rec ? rec : nullptr, ws.S, ws.dwh,
+        if (rt.dw_cols)
+            TRY(cu(launch_conv_dw_cols(gp, ni, C_out, c, rt.dw_S ? nullptr : rec, ws.S, ws.dwh,
                                        last ? ws.count : nullptr, qcoef, g_W, g.C, st)));
-        else if (ws.S)
+        else if (rt.dw_S)
             TRY(cu(launch_conv_dw_tma(gp, ni, C_out, c, ws.S, ws.dwh, last ? ws.count : nullptr, qcoef, g_W, g.C,
                                       st)));
         else
@@ -1192,6 +1217,24 @@ size_t dstd_conv_workspace_bytes(int B, int H, int W, int C_in, int C_out, int k
     size_t f = conv_fwd_layout(nullptr, pl, C_out, Mp, op_of(math)).bytes;
     size_t g = conv_bwd_layout(nullptr, pl, C_out, Mp, bwd_op_of(math), true).bytes;
     return f > g ? f : g;
+}
+
+int dstd_conv_route(int B, int H, int W, int C_in, int C_out, int k, int stride, int pad, const dstd_params *p,
+                    dstd_math math) {
+    TRY(check_params(p));
+    const int Mp = padded_M(p->M);
+    if (C_out < 1) return DSTD_E_INVALID;
+    if (math == DSTD_MATH_F32) return DSTD_E_UNSUPPORTED;
+    TRY(check_math(math, Mp));
+    ConvPlan pl;
+    TRY(conv_plan(B, H, W, C_in, k, stride, pad, Mp, true, C_out, &pl));
+    if (!conv_use_implicit(math, pl.g, C_out, Mp)) return 0;
+    const int ni = conv_impl_images(pl.g, C_out, Mp);
+    const ConvFwdRoute f = conv_fwd_route(pl.g, ni, C_out, Mp);
+    const ConvBwdRoute b = conv_bwd_route(pl.g, ni, C_out, Mp);
+    return DSTD_ROUTE_IMPLICIT | (f.S || f.rows ? DSTD_ROUTE_FUSED_SCAN : 0) | (f.rows ? DSTD_ROUTE_FWD_ROWS : 0) |
+           (f.S ? DSTD_ROUTE_FWD_BINNED : 0) | (b.ds_rows ? DSTD_ROUTE_DS_ROWS : 0) |
+           (b.dw_cols ? DSTD_ROUTE_DW_COLUMNS : 0) | (b.dw_S ? DSTD_ROUTE_DW_BINNED : 0);
 }
 
 int dstd_conv_fwd(const float *t_in, const float *W, int B, int H, int Wd, int C_in, int C_out, int k, int stride,
