@@ -730,13 +730,14 @@ struct ConvBwdRoute {
     bool ds_rows, ds_cb_inner;  // dS by source rows, and the order of its products
     bool dw_cols;               // dW by columns
     bool dw_S;                  // dW reads the binned input written out, else records
+    ConvDwColsSplit dw_split;   // of dW by columns
 };
 static ConvBwdRoute conv_bwd_route(const ConvGeom &g, int ni, int C_out, int Mp) {
     const ConvGeom gp = conv_padded(g);
-    ConvBwdRoute r{false, !conv_ds_row_boxes(gp, C_out, Mp), false, conv_dw_tma(g, C_out)};
+    ConvBwdRoute r{false, !conv_ds_row_boxes(gp, C_out, Mp), false, conv_dw_tma(g, C_out), {}};
     if (g_conv_operand_policy != 0) return r;
     r.ds_rows = conv_rows_ds_supported(gp, ni, C_out, Mp, r.ds_cb_inner);
-    r.dw_cols = r.dw_S && conv_dw_cols_supported(gp, C_out, Mp);
+    r.dw_cols = r.dw_S && conv_dw_cols_pick(gp, ni, C_out, Mp, g.C, r.dw_split);
     if (r.dw_cols && conv_dw_cols_records(C_out)) r.dw_S = false;
     return r;
 }
@@ -854,8 +855,8 @@ int conv_bwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
         }
         Timed tm(KK_GEMM_DW, st);
         if (rt.dw_cols)
-            TRY(cu(launch_conv_dw_cols(gp, ni, C_out, c, rt.dw_S ? nullptr : rec, ws.S, ws.dwh,
-                                       last ? ws.count : nullptr, qcoef, g_W, g.C, st)));
+            TRY(cu(launch_conv_dw_cols(gp, ni, C_out, c, rt.dw_split, rt.dw_S ? nullptr : rec, ws.S,
+                                       ws.dwh, last ? ws.count : nullptr, qcoef, g_W, g.C, st)));
         else if (rt.dw_S)
             TRY(cu(launch_conv_dw_tma(gp, ni, C_out, c, ws.S, ws.dwh, last ? ws.count : nullptr, qcoef, g_W, g.C,
                                       st)));

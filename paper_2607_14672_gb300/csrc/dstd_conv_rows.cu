@@ -1576,23 +1576,76 @@ cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifC
     return rows_launch<64, 1, false>(mA, mB, a, p, st);
 }
 
-// 3x3 layers at stride 1 with 64 output channels (1.1 to 1.4 times faster than a
-// box per tap, 0.97 on 3000 positions), and wider ones with 64 grid steps (128
-// -> 128 at 14 x 14: 1.37; 256 -> 256 at 7 x 7: 1.09). Wider ones with 32 grid
-// steps stay with a box per tap: a K step is then one position of 32, half of
-// whose MMA block (2, kw) is not used (1.07 at 64 input channels, 0.68 to 0.99
-// at 128 and more).
 bool conv_dw_cols_records(int C_out) { return C_out == 64; }
 
-bool conv_dw_cols_supported(const ConvGeom &g, int C_out, int Mp) {
-    return g.k == 3 && g.s == 1 && g.C % 64 == 0 &&
-           ((C_out == 64 && (Mp == 32 || Mp == 64)) || (C_out % 128 == 0 && Mp == 64));
+// The ranges of rows: the fewest rounds of tiles on the SMs x (rows + the cost
+// of a tile's epilogue, about two rows of 28 positions), but at least as many
+// as splits in k_conv_dw_tma where the chunk has that many rows, with 128
+// columns half as many again: the tensor core cuts its sums off, so the error
+// of a range grows with its length. With one round of tiles dW of 64 -> 64 at
+// 28 x 28 was 24e-6 off and of 128 -> 128 at 14 x 14 8e-6, against 16e-6 and
+// 2e-6 of that kernel.
+static ConvDwColsSplit dw_cols_split(const ConvGeom &g, int ni, int C_out) {
+    const int BN = C_out == 64 ? 64 : 128, ncb = g.C / 64, n_col = C_out / BN, rows = ni * g.Ho;
+    const int per = ncb * (BN == 64 ? 1 : 2) * n_col, sms = rows_num_sms();
+    const int G = BN == 64 ? 5 : 3, row_tiles = (9 * ncb + 1) / 2;
+    int least = (BN == 64 ? 2 : 3) * sms / ((row_tiles + G - 1) / G * n_col);
+    if (least > rows) least = rows;
+    const double tail = 56.0 / g.Wo;
+    double best = -1.0;
+    ConvDwColsSplit sp{1, 0};
+    for (int n = least < 1 ? 1 : least; n <= rows && (n <= least || n <= 4 * sms); ++n) {
+        const int rp = (rows + n - 1) / n, ns = (rows + rp - 1) / rp;
+        const double cost = (double)(((long long)per * ns + sms - 1) / sms) * (rp + tail);
+        if (best < 0.0 || cost < best) {
+            best = cost;
+            sp = ConvDwColsSplit{rp, per * ns};
+        }
+    }
+    return sp;
 }
 
-cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const uint2 *rec,
-                                const __nv_bfloat16 *S, const __nv_bfloat16 *dW_hat, const float *count, float qcoef, float *g_W, int C_t,
-                                cudaStream_t st) {
-    if (!conv_dw_cols_supported(g, C_out, c.Mp)) return cudaErrorInvalidConfiguration;
+// Shapes: 3x3 at stride 1, 64 output channels, or a multiple of 128 with 64
+// grid steps. (With 32 a K step of those is one position of 32, half of whose
+// MMA block (2, kw) is not used: 0.68 to 0.99 of the speed of a box per tap.)
+// Of those, where the kernel is expected to be the faster one. By columns it
+// pays for two more columns per row and for atomics per range, so it loses on
+// few positions and on narrow images, unless a single round of short rows does
+// it. Measured, a box per tap / by columns (with 64 output channels S or the
+// records included), us: 64 -> 64, M = 64: 12 images of 2 x 2 25 / 23, 250 of
+// 2 x 2 26 / 35, one of 28 x 28 26 / 39, 20 of 14 x 14 46 / 47, 82 of 14 x 14
+// 150 / 108, 82 of 28 x 28 520 / 349; 128 -> 64, M = 32: 40 of 10 x 10 49 / 63;
+// 128 -> 128: 12 of 2 x 2 23 / 16, 250 of 2 x 2 35 / 51, 20 of 14 x 14 64 / 82, 163 of
+// 14 x 14 480 / 414; 256 -> 256: 50 of 2 x 2 27 / 46, 82 of 14 x 14 841 / 756; 512 ->
+// 512: 62 of 4 x 4 213 / 241. The times are fitted as in conv_dw_tma_us (3% rms):
+// launch, a position of a row, a row's two more columns, a tile's epilogue; S
+// at 5.7 TB/s, the records at 2.5.
+// Over the fitted shapes the choice costs 0.3% against the better of the two.
+bool conv_dw_cols_pick(const ConvGeom &g, int ni, int C_out, int Mp, int C_t, ConvDwColsSplit &sp) {
+    if (g.k != 3 || g.s != 1 || g.C % 64 != 0) return false;
+    if (!(C_out == 64 && (Mp == 32 || Mp == 64)) && !(C_out % 128 == 0 && Mp == 64)) return false;
+    sp = dw_cols_split(g, ni, C_out);
+    struct Fit {
+        double launch, pos, row, epi;
+    };
+    const Fit f = C_out != 64 ? Fit{8.2, 0.403, 0.292, 6.40}
+                  : Mp == 64  ? Fit{9.2, 0.611, 0.513, 6.34}
+                  : C_t < 64  ? Fit{8.6, 0.489, 0.550, 6.16}   // (its generators have less to write)
+                              : Fit{8.8, 0.537, 0.631, 5.58};
+    const double rounds = (double)((sp.n_tiles + rows_num_sms() - 1) / rows_num_sms());
+    double cols = f.launch + rounds * (sp.rows_per * (g.Wo * f.pos + f.row) + f.epi);
+    double taps = conv_dw_tma_us(g, ni, C_out, Mp);
+    if (conv_dw_cols_records(C_out)) {
+        const double in_mb = 1e-6 * ni * g.H * g.W;
+        cols += 5.5 + in_mb * C_t * 12 * 0.405;
+        taps += 6.3 + in_mb * g.C * Mp * 2 * 0.177;
+    }
+    return cols < taps;
+}
+
+cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const ConvDwColsSplit &sp,
+                                const uint2 *rec, const __nv_bfloat16 *S, const __nv_bfloat16 *dW_hat,
+                                const float *count, float qcoef, float *g_W, int C_t, cudaStream_t st) {
     DwColsPlan p{};
     p.H = g.H;
     p.W = g.W;
@@ -1603,7 +1656,7 @@ cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifC
     p.pad = g.p;
     p.Mp = c.Mp;
     p.ncb = g.C / 64;
-    const int BN = C_out == 64 ? 64 : 128;
+    const int BN = C_out == 64 ? 64 : 128, sms = rows_num_sms();
     p.n_col = C_out / BN;
     p.rows = ni * g.Ho;
     if (p.rows == 0) return cudaSuccess;
@@ -1611,27 +1664,8 @@ cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifC
     p.g_W = g_W;
     p.count = count;
     p.qcoef = qcoef;
-    // ranges of rows: the fewest rounds of tiles on the SMs x (rows + the cost
-    // of a tile's epilogue, about two rows of 28 positions), but at least as
-    // many as splits in k_conv_dw_tma, with 128 columns half as many again: the
-    // tensor core cuts its sums off, so the error of a range grows with its
-    // length. With one round of tiles dW of 64 -> 64 at 28 x 28 was 24e-6 off and
-    // of 128 -> 128 at 14 x 14 8e-6, against 16e-6 and 2e-6 of that kernel.
-    const int per = p.ncb * (BN == 64 ? 1 : 2) * p.n_col, sms = rows_num_sms();
-    const int G = BN == 64 ? 5 : 3, row_tiles = (9 * p.ncb + 1) / 2;
-    int least = (BN == 64 ? 2 : 3) * sms / ((row_tiles + G - 1) / G * p.n_col);
-    if (least > p.rows) least = p.rows;
-    const double tail = 56.0 / g.Wo;
-    double best = -1.0;
-    for (int n = least < 1 ? 1 : least; n <= p.rows && (n <= least || n <= 4 * sms); ++n) {
-        const int rp = (p.rows + n - 1) / n, ns = (p.rows + rp - 1) / rp;
-        const double cost = (double)(((long long)per * ns + sms - 1) / sms) * (rp + tail);
-        if (best < 0.0 || cost < best) {
-            best = cost;
-            p.rows_per = rp;
-            p.n_tiles = per * ns;
-        }
-    }
+    p.rows_per = sp.rows_per;
+    p.n_tiles = sp.n_tiles;
     const int slot = (BN == 64 ? DwCols<64>::SLOT_BOXES : DwCols<128>::SLOT_BOXES) * c.Mp * 128;
     const int extra = BN == 64 ? DwCols<64>::EXTRA : DwCols<128>::EXTRA;
     p.ring = (ROWS_SMEM_MAX - extra) / slot;

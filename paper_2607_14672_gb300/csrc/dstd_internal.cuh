@@ -516,13 +516,19 @@ cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifC
                                 const __nv_bfloat16 *dW_hat, const __nv_bfloat16 *Wt, const float *t_in, float *g_t_in, int C_t, cudaStream_t st);
 // dW of 3x3 layers at stride 1, each column of S taken once per channel block
 // (same file; as launch_conv_dw_tma): generated from the records [ni H W][C_t]
-// where conv_dw_cols_records says so, else (rec null) read from S
-bool conv_dw_cols_supported(const ConvGeom &g, int C_out, int Mp);
+// where conv_dw_cols_records says so, else (rec null) read from S. pick:
+// whether it is the faster one, and how its rows are split
+struct ConvDwColsSplit {
+    int rows_per, n_tiles;  // output rows of a range, and ranges x tiles of one
+};
+bool conv_dw_cols_pick(const ConvGeom &g, int ni, int C_out, int Mp, int C_t, ConvDwColsSplit &sp);
 bool conv_dw_cols_records(int C_out);
-cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const uint2 *rec,
-                                const __nv_bfloat16 *S, const __nv_bfloat16 *dW_hat, const float *count, float qcoef, float *g_W, int C_t,
-                                cudaStream_t st);
+cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const ConvDwColsSplit &sp,
+                                const uint2 *rec, const __nv_bfloat16 *S, const __nv_bfloat16 *dW_hat,
+                                const float *count, float qcoef, float *g_W, int C_t, cudaStream_t st);
 cudaError_t conv_rows_status_read(unsigned int *out, int clear);
+// expected time of launch_conv_dw_tma (without writing S)
+double conv_dw_tma_us(const ConvGeom &g, int ni, int C_out, int Mp);
 // dW from S and dw^ (added into g_W as for launch_conv_dw_gen)
 // (g.C may be the padded channel count; g_W is [C_out][k k C_t])
 cudaError_t launch_conv_dw_tma(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *S,

@@ -4,7 +4,11 @@ to check the kernels by source rows against the one-row-at-a-time kernels do tak
 Forward by rows: 64 output channels, one block of 64 input channels (or fewer, padded), stride 1, filters above 1x1,
 300 output positions per SM. dS by rows: one block of input channels, 20 input positions per SM, at most eight output
 rows in flight (four at stride 2). Forward results are equal bit for bit, input-time gradients to 1e-5 relative L2
-(the two bins of an input may be added in either order), as in test_gpu_conv_rows.py."""
+(the two bins of an input may be added in either order), as in test_gpu_conv_rows.py.
+
+dW by columns: 3x3 at stride 1, 64 output channels, or a multiple of 128 with 64 grid steps, on the side of the
+measured crossing where it is the faster one. Weight gradients are fp32 sums in another order: 2e-5 relative L2, as in
+test_gpu_conv_rows.py."""
 
 import math
 import os
@@ -34,6 +38,22 @@ LARGE = [
     (14, 14, 128, 64, 3, 1, 1, 64, (1.0, 0.25), set()),
 ]
 ROWS = {"fwd_rows", "ds_rows"}
+
+# B, H, W, C_in, C_out, pad, M of 3x3 layers at stride 1: clearly faster by columns ...
+COLUMNS = [
+    (256, 28, 28, 64, 64, 1, 64), (256, 28, 28, 3, 64, 1, 64), (82, 14, 14, 64, 64, 1, 64), (82, 7, 7, 256, 64, 1, 64),
+    (256, 14, 14, 128, 128, 1, 64), (164, 14, 14, 256, 256, 1, 64),
+    (12, 2, 2, 64, 64, 1, 32), (25, 1, 1, 64, 64, 1, 32), (12, 2, 2, 64, 64, 1, 64),
+    (3, 4, 3, 192, 64, 1, 20), (2, 6, 5, 5, 64, 0, 32), (12, 2, 2, 128, 128, 1, 64), (25, 1, 1, 128, 128, 1, 64),
+    (2, 3, 4, 64, 128, 1, 50), (3, 2, 2, 128, 256, 2, 33), (800, 5, 4, 64, 64, 2, 40), (700, 9, 9, 64, 128, 0, 64),
+]
+# ... and clearly slower
+TAPS = [
+    (250, 2, 2, 64, 64, 1, 64), (1, 28, 28, 64, 64, 1, 64), (1, 28, 28, 128, 64, 1, 64), (111, 3, 3, 64, 64, 1, 64),
+    (40, 10, 10, 128, 64, 1, 32), (40, 10, 10, 256, 64, 1, 32), (50, 2, 2, 256, 256, 1, 64), (12, 2, 2, 512, 512, 1, 64),
+    (62, 4, 4, 512, 512, 1, 64), (20, 14, 14, 128, 128, 1, 64), (1000, 2, 2, 128, 128, 1, 64),
+    (256, 14, 14, 128, 128, 1, 32),
+]
 
 
 @pytest.fixture(scope="module")
@@ -85,6 +105,33 @@ def test_refused_and_other_paths(lib):
         with pytest.raises(dstd.DstdError) as e:
             dstd.conv_route(*bad)
         assert e.value.code == code
+
+
+def dw_case(c):
+    B, H, W, C, O, pad, M = c
+    return H, W, C, O, 3, 1, pad, M, (1.0, 0.25) if M > 32 else (INF, INF)
+
+
+@pytest.mark.parametrize("c", COLUMNS + TAPS, ids=lambda c: "-".join(str(x) for x in c))
+def test_columns_where_they_are_faster(lib, c):
+    r = route(c[0], dw_case(c))
+    assert ("dw_columns" in r) == (c in COLUMNS)
+    assert ("dw_binned" in r) == (c not in COLUMNS or c[4] != 64)
+    assert "dw_columns" not in route(c[0], dw_case(c), policy=2)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("c", [c for c in COLUMNS if c[0] * c[1] * c[2] < 60000], ids=lambda c: "-".join(str(x) for x in c))
+def test_columns_are_taken_and_match(lib, c):
+    import torch
+    from paper_2607_14672_gb300 import dstd
+    from test_gpu_conv_rows import rel, run
+    dstd.device_status(clear=True)
+    case = dw_case(c)
+    assert "dw_columns" in route(c[0], case) and "dw_columns" not in route(c[0], case, policy=2)
+    a, b = run(c[0], *case, policy=0), run(c[0], *case, policy=2)
+    assert torch.equal(a[0], b[0]) and (b[4] != 0).any()
+    assert rel(a[4], b[4]) <= 2e-5
 
 
 @pytest.mark.gpu
