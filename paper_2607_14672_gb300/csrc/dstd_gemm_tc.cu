@@ -204,29 +204,93 @@ struct TileInfo {
     int row0, col0, kt0, nkt, split;
 };
 
-// Order of the output tiles: bands of `band` row tiles, down the rows of a
-// band first, then across its columns. The tiles that run at one time so
-// cover a block of the output about as high as it is wide, whose operand rows
-// stay in L2 for the whole K loop. Down all the rows first, the operand of a
-// 16384-row side (512 MB) came from HBM once per column of tiles, and that
-// bound the contraction (16384 wide, M = 128, bf16: 8.8 ms, 0.51 of the peak;
-// in bands 7.1 ms on pairs, 6.7 ms on single CTAs, 0.64 and 0.67).
-__device__ __forceinline__ void tile_order(int rem, int n_row, int n_col, int band, int &rt, int &ct) {
-    const int per = band * n_col;
-    const int bd = rem / per, r = rem - bd * per;
-    const int left = n_row - bd * band, h = left < band ? left : band;
+// Order of the output tiles: n bands of `high` row tiles (the last one what is
+// left), down the rows of a band first, then across its columns. The tiles that
+// run at one time so cover a block of the output about as high as it is wide,
+// whose operand rows stay in L2 for the whole K loop. Down all the rows first,
+// the operand of a 16384-row side (512 MB) came from HBM once per column of
+// tiles, and that bound the contraction (16384 wide, M = 128, bf16: 8.8 ms, 0.51
+// of the peak; in bands 7.1 ms on pairs, 6.7 ms on single CTAs, 0.64 and 0.67).
+struct Bands {
+    int high, n;
+};
+__device__ __forceinline__ void tile_order(int rem, int n_row, int n_col, Bands b, int &rt, int &ct) {
+    const int per = b.high * n_col;
+    int bd = rem / per;
+    if (bd >= b.n) bd = b.n - 1;
+    const int r = rem - bd * per, h = bd == b.n - 1 ? n_row - bd * b.high : b.high;
     ct = r / h;
-    rt = bd * band + (r - ct * h);
+    rt = bd * b.high + (r - ct * h);
 }
 constexpr int BAND = 12;      // 152 CTAs: 12 x 12.7 tiles of 128 x 128
 constexpr int BAND_PAIR = 6;  // 76 SM pairs: 6 x 12.7 tiles of 256 x 128
 
-__device__ __forceinline__ TileInfo tile_info(int t, int n_row, int n_col, int ktiles, int kt_per_split, int BNv) {
+// The bands of an R x Cn x K product with operands of `bytes` per element (all
+// parts). Every band reads the column operand again, from HBM where it is
+// larger than L2 can keep beside the rest, so:
+//   - a single row tile left over joins the band above it: 13 row tiles of 128
+//     (1600 rows) in 12 + 1 read 131 MB of columns twice (x3, 32000 columns, K =
+//     1024: 259 us, in one band 241; bf16 dW of 1600 x 8192, K = 4096: 116, 110);
+//   - on pairs all rows are one band where their operand stays in L2 by itself
+//     (up to 52 MB) and there are at least 16 column tiles (bf16, 8192 x 8192,
+//     K = 2048: 219 us in bands, 209 in one; 4096 x 32000, K = 3000: 756, 730; with 67
+//     MB of rows, 8192 x 1600, K = 4096: 90 in bands, 93 in one). On single CTAs bands
+//     are the faster order there too (x3, 8192 x 8192, K = 512: 171 us, 200 in one).
+static Bands pick_bands(int n_row, int n_col, int K, int bytes, bool pair) {
+    const int high = pair ? BAND_PAIR : BAND;
+    if (n_row <= high + 1) return Bands{n_row, 1};
+    if (pair && n_col >= 16 && (double)n_row * 256 * K * bytes <= 52e6) return Bands{n_row, 1};
+    return Bands{high, (n_row + high - 2) / high};
+}
+
+// n / d for 0 <= n < 2^31 by a multiplication and a shift. In dS on single CTAs,
+// where a tile is often one or two K slices long, the divisions of its place in
+// the order count (every role works out every tile): 128 -> 48 conv layer by im2col
+// 200 us with divisions, 192 without. (The other kernels keep the divisions: with
+// the multipliers the bf16 Store kernel came out 3 to 5% slower.)
+struct FastDiv {
+    int d;
+    uint32_t mul, shift;
+    __device__ __forceinline__ int div(int n) const {
+        return (int)((__umulhi((uint32_t)n, mul) + (uint32_t)n) >> shift);
+    }
+};
+static FastDiv fast_div(int d) {
+    uint32_t s = 0;
+    while ((1ull << s) < (unsigned long long)d) ++s;
+    return FastDiv{d, (uint32_t)((((1ull << s) - (unsigned long long)d) << 32) / (unsigned long long)d + 1), s};
+}
+
+// the same order for single CTAs, over the K splits: divisors are the tiles of a
+// split and of a band, and the rows of a band and of the last one
+struct TileOrder {
+    int n_row, n_col;
+    Bands b;
+    FastDiv tiles, band, by_high, by_last;
+};
+static TileOrder tile_order_of(int n_row, int n_col, Bands b) {
+    return TileOrder{n_row, n_col, b, fast_div(n_row * n_col), fast_div(b.high * n_col), fast_div(b.high),
+                     fast_div(n_row - (b.n - 1) * b.high)};
+}
+
+template <bool FAST>
+__device__ __forceinline__ TileInfo tile_info(int t, const TileOrder &o, int ktiles, int kt_per_split, int BNv) {
     TileInfo ti;
-    const int per_split = n_row * n_col;
-    ti.split = t / per_split;
     int rt, ct;
-    tile_order(t - ti.split * per_split, n_row, n_col, BAND, rt, ct);
+    if (FAST) {
+        ti.split = o.tiles.div(t);
+        const int rem = t - ti.split * o.tiles.d;
+        int bd = o.band.div(rem);
+        const bool last = bd >= o.b.n - 1;
+        if (last) bd = o.b.n - 1;
+        const int r = rem - bd * o.band.d;
+        ct = last ? o.by_last.div(r) : o.by_high.div(r);
+        rt = bd * o.b.high + r - ct * (last ? o.by_last.d : o.b.high);
+    } else {
+        const int per_split = o.n_row * o.n_col;
+        ti.split = t / per_split;
+        tile_order(t - ti.split * per_split, o.n_row, o.n_col, o.b, rt, ct);
+    }
     ti.row0 = rt * BM;
     ti.col0 = ct * BNv;
     ti.kt0 = ti.split * kt_per_split;
@@ -239,8 +303,9 @@ template <int NPASS, int BN, int EPI, bool F16, bool BMN>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ CUtensorMap mA_lo,
               const __grid_constant__ CUtensorMap mB_hi, const __grid_constant__ CUtensorMap mB_lo, int R, int Cn,
-              int ktiles, int kt_per_split, int n_row, int n_col, int n_split, TcEpiArgs args) {
+              int ktiles, int kt_per_split, const __grid_constant__ TileOrder order, int n_split, TcEpiArgs args) {
     using C = Cfg<NPASS, BN>;
+    constexpr bool FAST = EPI == (int)Epi::GradT;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + C::STAGES * C::STAGE);
@@ -250,7 +315,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ntiles = n_row * n_col * n_split;
+    const int ntiles = order.n_row * order.n_col * n_split;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::STAGES; ++s) {
@@ -274,7 +339,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             uint32_t it = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const TileInfo ti = tile_info(t, n_row, n_col, ktiles, kt_per_split, BN);
+                const TileInfo ti = tile_info<FAST>(t, order, ktiles, kt_per_split, BN);
                 for (int i = 0; i < ti.nkt; ++i, ++it) {
                     const int s = it % C::STAGES;
                     const uint32_t ph = (it / C::STAGES) & 1u;
@@ -312,7 +377,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             uint32_t it = 0, j = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++j) {
-                const TileInfo ti = tile_info(t, n_row, n_col, ktiles, kt_per_split, BN);
+                const TileInfo ti = tile_info<FAST>(t, order, ktiles, kt_per_split, BN);
                 if (j > 0) {
                     // the epilogue of the previous tile has taken the accumulator
                     if (!mbar_wait(acc_empty, (j - 1) & 1u)) {
@@ -368,7 +433,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (c_hi > BN) c_hi = BN;
         uint32_t j = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++j) {
-            const TileInfo ti = tile_info(t, n_row, n_col, ktiles, kt_per_split, BN);
+            const TileInfo ti = tile_info<FAST>(t, order, ktiles, kt_per_split, BN);
             if (!mbar_wait_sleep(acc_full, j & 1u)) {
                 set_status(STATUS_TIMEOUT);
                 break;
@@ -567,7 +632,7 @@ template <int NPASS, bool F16, int EPI, bool BMN>
 __global__ void __launch_bounds__(pair_threads<NPASS>(), 1)
     k_tc_gemm_pair(const __grid_constant__ CUtensorMap mA_hi, const __grid_constant__ CUtensorMap mA_lo,
                    const __grid_constant__ CUtensorMap mB_hi, const __grid_constant__ CUtensorMap mB_lo, int R,
-                   int Cn, int ktiles, int n_row, int n_col, TcEpiArgs args) {
+                   int Cn, int ktiles, int n_row, int n_col, Bands bands, TcEpiArgs args) {
     using C = Cfg2<NPASS>;
     constexpr int MW = pair_mma_warps<NPASS>();
     static_assert(!BMN || NPASS == 1, "the MN-major B of the pair kernel: bf16 mode only");
@@ -610,7 +675,7 @@ __global__ void __launch_bounds__(pair_threads<NPASS>(), 1)
             bool ok = true;
             for (int t = cid; t < ntiles && ok; t += ncl) {
                 int rt, ct;
-                tile_order(t, n_row, n_col, BAND_PAIR, rt, ct);
+                tile_order(t, n_row, n_col, bands, rt, ct);
                 const int row0 = rt * (2 * BM2) + rank * BM2;
                 const int brow0 = ct * (2 * BNH) + rank * BNH;
                 for (int i = 0; i < ktiles; ++i, ++it) {
@@ -763,7 +828,7 @@ __global__ void __launch_bounds__(pair_threads<NPASS>(), 1)
         uint32_t j = 0;
         for (int t = cid; t < ntiles; t += ncl, ++j) {
             int rt, ct;
-            tile_order(t, n_row, n_col, BAND_PAIR, rt, ct);
+            tile_order(t, n_row, n_col, bands, rt, ct);
             const int row = rt * (2 * BM2) + rank * BM2 + quarter * 32 + lane;
             const int col0 = ct * C::BNP + (EPI == (int)Epi::Store ? c_lo : 0);
             if (!mbar_wait_cluster(acc_full, j & 1u, true)) {
@@ -883,10 +948,11 @@ static cudaError_t launch_one(const CUtensorMap &a_hi, const CUtensorMap &a_lo, 
     const int ktiles = (K + BK - 1) / BK;
     const int per = (ktiles + splits - 1) / splits;
     const int n_row = (R + BM - 1) / BM, n_col = (Cn + BN - 1) / BN;
+    const TileOrder order = tile_order_of(n_row, n_col, pick_bands(n_row, n_col, K, NPASS == 3 ? 4 : 2, false));
     const long long ntiles = (long long)n_row * n_col * splits;
     const int grid = (int)(ntiles < num_sms() ? ntiles : num_sms());
     k_tc_gemm<NPASS, BN, EPI, F16, BMN><<<grid, NTHREADS, C::SMEM, st>>>(a_hi, a_lo, b_hi, b_lo, R, Cn, ktiles, per,
-                                                                            n_row, n_col, splits, args);
+                                                                            order, splits, args);
     return cudaGetLastError();
 }
 
@@ -952,7 +1018,8 @@ static cudaError_t launch_pair(const CUtensorMap &a_hi, const CUtensorMap &a_lo,
     if (resident < 1) return cudaErrorInvalidConfiguration;
     const int pairs = (int)(ntiles < resident ? ntiles : resident);
     cfg.gridDim = dim3(2 * pairs);
-    return cudaLaunchKernelEx(&cfg, kern, a_hi, a_lo, b_hi, b_lo, R, Cn, ktiles, n_row, n_col, args);
+    const Bands bands = pick_bands(n_row, n_col, K, NPASS == 3 ? 4 : 2, true);
+    return cudaLaunchKernelEx(&cfg, kern, a_hi, a_lo, b_hi, b_lo, R, Cn, ktiles, n_row, n_col, bands, args);
 }
 }  // namespace tc
 
