@@ -183,37 +183,6 @@ __device__ __forceinline__ uint32_t row_plan(const Item<FWD> &w, const RowsPlan 
            ((q & (uint32_t)(NA - 1)) << 4) | ((((q / NA) & 1u) ^ 1u) << 7);
 }
 
-// The recurrence over one bin, (v, I) -> I0 = I + w^_m, v' = rv v + KD I0,
-// I' = rI I0, with every rounding spelled out: spike times near a tangential
-// crossing depend on the last bit, and scan_walk, whose results these are bit
-// for bit, has rI I0 fused into the next bin's addition where its unrolling let
-// the compiler do so (within a group of four quiet bins, and within the whole
-// groups of four of the walk to a flagged bin).
-__device__ __forceinline__ float walk_v(const LifConst &c, float v, float I0) {
-    return fmaf(c.KD, I0, __fmul_rn(c.rv, v));
-}
-// state at bin k0 + n from the state at k0 (n < 8)
-__device__ __forceinline__ void walk_to(const LifConst &c, const float *row, int n, float &v, float &I) {
-    int k = 0;
-    if (n & 4) {
-        float i0 = __fadd_rn(I, row[0]);
-        v = walk_v(c, v, i0);
-#pragma unroll
-        for (int u = 1; u < 4; ++u) {
-            i0 = fmaf(c.rI, i0, row[u]);
-            v = walk_v(c, v, i0);
-        }
-        I = __fmul_rn(c.rI, i0);
-        k = 4;
-    }
-#pragma unroll 1
-    for (; k < n; ++k) {
-        const float i0 = __fadd_rn(I, row[k]);
-        v = walk_v(c, v, i0);
-        I = __fmul_rn(c.rI, i0);
-    }
-}
-
 // four bins in the bare recurrence: rounding as the group took it in the pass
 // over the bins (fused or not, see scan_walk)
 __device__ __forceinline__ void walk_group(const LifConst &c, const float *x, bool fused, float &v, float &I) {
@@ -252,14 +221,13 @@ __device__ __forceinline__ void walk_group(const LifConst &c, const float *x, bo
 // cache (64 -> 64 at 28 x 28, B = 256, M = 64: 3.2 ms against 2.2 ms); where it
 // runs alone, in the dense scan, unrolled is the faster one (16384 wide, M =
 // 128: 295 against 320 us).
-__device__ __forceinline__ bool walk_rolled(const LifConst &c, const float *row, int m0, int mend, float &v, float &I,
-                                            ScanState &st) {
+__device__ __forceinline__ bool walk_rolled(unsigned lanes, const LifConst &c, const float *row, int m0, int mend,
+                                            float &v, float &I, ScanState &st) {
     float cv = v, cI = I;             // state at the start of the current eight bins
     float kv = v, kI = I;             // and of the first flagged eight, kb
     int kb = -1;
     uint32_t mask = 0u, fused = 0u;   // flagged bins; groups that took the bare recurrence
     bool looking = true;
-    const unsigned lanes = __activemask();
     const float vlow = c.vth * 0.99999f, vhigh = c.vth * 1.00001f;
 #pragma unroll 1
     for (int g = 0; g < 32; g += 4) {
@@ -274,7 +242,7 @@ __device__ __forceinline__ bool walk_rolled(const LifConst &c, const float *row,
                            fmaxf(xs[3], 0.0f);
         const bool quiet = fmaf(ipos, c.Kmax4, fmaxf(v, 0.0f)) < vlow;
         if (__all_sync(lanes, quiet)) {
-            walk_group(c, xs, true, v, I);
+            walk_fused<4>(c, xs, v, I);
             fused |= 1u << (g >> 2);
         } else {
             float vs[5], I0[4], In[4];
@@ -323,7 +291,7 @@ __device__ __forceinline__ bool walk_rolled(const LifConst &c, const float *row,
             walk_group(c, row + kb * 8 + 4, (fused >> (kb * 2 + 1)) & 1u, kv, kI);
         }
         float vw = kv, Iw = kI;
-        walk_to(c, row + kb * 8, m & 7, vw, Iw);
+        walk_to<false>(c, row + kb * 8, m & 7, vw, Iw);
         const float I0 = __fadd_rn(Iw, row[m]);
         const float ve = walk_v(c, vw, I0);
         float hi = -1.0f;
@@ -794,11 +762,13 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                 }
                 h = stb[(cnt & 1u) * 32 + lane];
             }
-            if (on && __float_as_int(h.x) < 0) {
+            const bool walks = on && __float_as_int(h.x) < 0;
+            const unsigned lanes = __ballot_sync(0xffffffffu, walks);
+            if (walks) {
                 ScanState st;
                 scan_reset(st, a.c.M);
                 const int m0 = upper ? 32 : 0, mend = two && !upper ? 32 : a.c.M - m0;
-                if (walk_rolled(a.c, tb + lane * EPI_LDF, m0, mend, h.y, h.z, st))
+                if (walk_rolled(lanes, a.c, tb + lane * EPI_LDF, m0, mend, h.y, h.z, st))
                     h = make_float4(__int_as_float(st.q), st.v0, st.I0, st.hi);
             }
             int f_pos = on ? pos : -1, f_ch = ch;  // the neuron to solve now

@@ -704,9 +704,11 @@ __global__ void __launch_bounds__(CONV_THREADS, 1)
                     ScanState st;
                     scan_reset(st, a.c.M);
                     float vv = 0.f, I = 0.f;
+                    bool hit = false;
                     for (int m0 = 0; m0 < a.c.M; m0 += 32) {
                         const int mend = (a.c.M - m0) < 32 ? (a.c.M - m0) : 32;
-                        if (scan_walk<32, !TIGHT>(a.c, row + m0, m0, mend, vv, I, st)) break;
+                        const unsigned lanes = __ballot_sync(0xffffffffu, !hit);
+                        if (!hit) hit = scan_walk<32, !TIGHT, false>(lanes, a.c, row + m0, m0, mend, vv, I, st);
                     }
                     scan_finish(a.c, st);
                     finish_neuron(a.c, st, p, ct * BN + (r * qpp + wip) * 32 + lane, a.C_out, a.rowsum, a.t_out,

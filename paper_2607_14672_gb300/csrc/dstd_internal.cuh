@@ -278,16 +278,51 @@ static __device__ __noinline__ float interior_test(float av, float aI, float lam
     return interval_test(av, aI, lam, lam_zero, rI, dt, vth, v0, I0, ve);
 }
 
-// One interval of the walk, with explicit fma so that the fast pass and the
-// exact pass round alike: the end state and the two flags.
+// The recurrence over one bin, (v, I) -> I0 = I + w^_m, v' = rv v + KD I0,
+// I' = rI I0, with every rounding spelled out: spike times near a tangential
+// crossing depend on the last bit.
+__device__ __forceinline__ float walk_v(const LifConst &c, float v, float I0) {
+    return fmaf(c.KD, I0, __fmul_rn(c.rv, v));
+}
+// N bins of it in which rI I0 goes into the next bin's addition in one
+// rounding (the last I' is rounded by itself)
+template <int N>
+__device__ __forceinline__ void walk_fused(const LifConst &c, const float *x, float &v, float &I) {
+    float i0 = __fadd_rn(I, x[0]);
+    v = walk_v(c, v, i0);
+#pragma unroll
+    for (int u = 1; u < N; ++u) {
+        i0 = fmaf(c.rI, i0, x[u]);
+        v = walk_v(c, v, i0);
+    }
+    I = __fmul_rn(c.rI, i0);
+}
+// The state n < 8 bins on, on the way to a flagged bin: four bins fused, then
+// two (PAIR) and one, or one by one.
+template <bool PAIR>
+__device__ __forceinline__ void walk_to(const LifConst &c, const float *row, int n, float &v, float &I) {
+    int k = 0;
+    if (n & 4) {
+        walk_fused<4>(c, row, v, I);
+        k = 4;
+    }
+    if (PAIR && (n & 2)) {
+        walk_fused<2>(c, row + k, v, I);
+        k += 2;
+    }
+#pragma unroll 1
+    for (; k < n; ++k) walk_fused<1>(c, row + k, v, I);
+}
+
+// One interval of the walk: the end state and the two flags.
 struct BinStep {
     float ve, In;
     bool endp, peak;
 };
 __device__ __forceinline__ BinStep bin_step(const LifConst &c, float v, float I0) {
     BinStep r;
-    r.ve = fmaf(c.KD, I0, c.rv * v);
-    r.In = c.rI * I0;
+    r.ve = walk_v(c, v, I0);
+    r.In = __fmul_rn(c.rI, I0);
     r.endp = r.ve >= c.vth;
     r.peak = (fmaf(-c.av, v, I0) > 0.0f) & (fmaf(-c.av, r.ve, r.In) < 0.0f) &
              (fmaf(fmaxf(I0, 0.0f), c.Kmax, fmaxf(v, 0.0f)) >= c.vth);
@@ -298,15 +333,24 @@ __device__ __forceinline__ BinStep bin_step(const LifConst &c, float v, float I0
 // values sit in row[0 .. SUB) (shared memory, zero past mend; 16-byte
 // aligned when VEC, read as float4), starting from the state (v, I) at T_m0.
 // On a spike, fills st (bin, state at its start, bracket end) and returns
-// true; otherwise leaves (v, I) at the end of the block.
-template <int SUB, bool VEC = true>
-__device__ __forceinline__ bool scan_walk(const LifConst &c, const float *row, int m0, int mend, float &v, float &I,
-                                          ScanState &st) {
+// true; otherwise leaves (v, I) at the end of the block. lanes: the lanes of
+// the warp that make this call together.
+//
+// The state's last bit depends on the path: a group of four bins in which
+// every lane is quiet takes rI I0 into the next addition in one rounding, the
+// flagged pass rounds it first, and the walk to a flagged bin rounds as
+// walk_to does. So a neuron's last bit can depend on the neurons beside it in
+// the warp. One rounding on every path would end that, but it moves neurons
+// that only just reach the threshold, whose gradients have 1 / v' (dW of 64 ->
+// 64 at 28 x 28, B = 256: by 9% in norm); so the roundings are written out as
+// they have been, for every kernel that walks (PAIR: the dense layers').
+template <int SUB, bool VEC, bool PAIR>
+__device__ __forceinline__ bool scan_walk(unsigned lanes, const LifConst &c, const float *row, int m0, int mend,
+                                          float &v, float &I, ScanState &st) {
     static_assert(SUB % 8 == 0 && SUB <= 32, "blocks of 8, 16 or 32 bins");
     constexpr int NCK = SUB / 8;  // kept states per block
     float kv[NCK], kI[NCK];
     uint32_t mask = 0u;
-    const unsigned lanes = __activemask();
 #pragma unroll
     for (int g = 0; g < SUB; g += 4) {
         if ((g & 7) == 0) {
@@ -329,19 +373,13 @@ __device__ __forceinline__ bool scan_walk(const LifConst &c, const float *row, i
                            fmaxf(xs[3], 0.0f);
         const bool quiet = fmaf(ipos, c.Kmax4, fmaxf(v, 0.0f)) < c.vth * 0.99999f;
         // one path per group for the whole warp: the flagged pass (its flags
-        // kept only where the bound is not met) unless every lane is quiet;
-        // both passes round alike, so the state does not depend on the path
+        // kept only where the bound is not met) unless every lane is quiet
         if (__all_sync(lanes, quiet)) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float I0 = I + xs[u];
-                v = fmaf(c.KD, I0, c.rv * v);
-                I = c.rI * I0;
-            }
+            walk_fused<4>(c, xs, v, I);
         } else {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const BinStep r = bin_step(c, v, I + xs[u]);
+                const BinStep r = bin_step(c, v, __fadd_rn(I, xs[u]));
                 if (!quiet && (r.endp | r.peak)) mask |= 1u << (g + u);
                 v = r.ve;
                 I = r.In;
@@ -359,12 +397,8 @@ __device__ __forceinline__ bool scan_walk(const LifConst &c, const float *row, i
             vw = (gk == k) ? kv[k] : vw;
             Iw = (gk == k) ? kI[k] : Iw;
         }
-        for (int k = gk * 8; k < m; ++k) {
-            const BinStep r = bin_step(c, vw, Iw + row[k]);
-            vw = r.ve;
-            Iw = r.In;
-        }
-        const float I0 = Iw + row[m];
+        walk_to<PAIR>(c, row + gk * 8, m & 7, vw, Iw);
+        const float I0 = __fadd_rn(Iw, row[m]);
         const BinStep r = bin_step(c, vw, I0);
         float hi = -1.0f;
         if (r.endp) hi = c.dt;

@@ -931,7 +931,10 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_scan_solve(const float *__r
         ScanState st;
         scan_reset(st, c.M);
         float v = 0.f, I = 0.f;
-        for (int m0 = 0; m0 < c.M && st.q == c.M; m0 += SUB) {
+        // lanes of this warp with a neuron that has not fired yet
+        const long long left = n - (idx - (threadIdx.x & 31));
+        unsigned lanes = left >= 32 ? 0xffffffffu : (1u << (int)left) - 1u;
+        for (int m0 = 0; m0 < c.M; m0 += SUB) {
             const int mend = (c.M - m0) < SUB ? (c.M - m0) : SUB;
             if (VEC && mend == SUB) {
 #pragma unroll
@@ -943,7 +946,9 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_scan_solve(const float *__r
 #pragma unroll
                 for (int j = 0; j < SUB; ++j) row[j] = (j < mend) ? __ldg(w + (m0 + j) * sm) * sc : 0.0f;
             }
-            if (scan_walk<SUB>(c, row, m0, mend, v, I, st)) break;
+            const bool hit = scan_walk<SUB, true, true>(lanes, c, row, m0, mend, v, I, st);
+            lanes = __ballot_sync(lanes, !hit);
+            if (hit) break;
         }
         scan_finish(c, st);
         finish_neuron(c, st, b, i, N, rowsum, t_out, q, s, vdot, acc);
@@ -1164,9 +1169,12 @@ __global__ void __launch_bounds__(NARROW_FWD_THREADS) k_narrow_fwd(const float *
         ScanState st;
         scan_reset(st, c.M);
         float v = 0.f, I = 0.f;
+        unsigned lanes = N_out >= 32 ? 0xffffffffu : (1u << N_out) - 1u;  // neurons that have not fired yet
         for (int m0 = 0; m0 < c.M; m0 += SUB) {
             const int mend = (c.M - m0) < SUB ? (c.M - m0) : SUB;
-            if (scan_walk<SUB>(c, acc + i * c.Mp + m0, m0, mend, v, I, st)) break;
+            const bool hit = scan_walk<SUB, true, true>(lanes, c, acc + i * c.Mp + m0, m0, mend, v, I, st);
+            lanes = __ballot_sync(lanes, !hit);
+            if (hit) break;
         }
         scan_finish(c, st);
         finish_neuron(c, st, b, i, N_out, rsum, t_out, q, s, vdot, pacc);
