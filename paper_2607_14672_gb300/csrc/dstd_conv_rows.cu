@@ -1432,7 +1432,7 @@ bool rows_plan(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_i
 template <int BN, int NT, bool FWD, int SLOTS>
 cudaError_t rows_launch_slots(const CUtensorMap &mA, const CUtensorMap &mB, const RowsArgs &a, const RowsPlan &p,
                         cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_rows<BN, NT, FWD, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+    cudaError_t e = allow_smem<k_conv_rows<BN, NT, FWD, SLOTS>>(p.smem);
     if (e != cudaSuccess) return e;
     const int grid = p.n_items < rows_num_sms() ? p.n_items : rows_num_sms();
     k_conv_rows<BN, NT, FWD, SLOTS><<<grid, Roles<BN, NT, FWD>::threads(p.nset), p.smem, st>>>(mA, mB, a, p);
@@ -1649,11 +1649,11 @@ cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifC
     const int smem = p.ring * slot + extra;
     const int grid = p.n_tiles < sms ? p.n_tiles : sms;
     if (BN == 64) {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_dw_cols<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = allow_smem<k_conv_dw_cols<64>>(smem);
         if (e != cudaSuccess) return e;
         k_conv_dw_cols<64><<<grid, DwCols<64>::THREADS, smem, st>>>(mS0, mS1, mD, p);
     } else {
-        cudaError_t e = cudaFuncSetAttribute(k_conv_dw_cols<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = allow_smem<k_conv_dw_cols<128>>(smem);
         if (e != cudaSuccess) return e;
         k_conv_dw_cols<128><<<grid, DwCols<128>::THREADS, smem, st>>>(mS0, mS1, mD, p);
     }

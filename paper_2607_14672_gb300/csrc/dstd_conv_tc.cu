@@ -1910,7 +1910,7 @@ static cudaError_t launch_fwd_gen_bn(const uint2 *rec, const CUtensorMap &mB, Co
     if (nst < FWD_GEN_GROUPS) return cudaErrorInvalidConfiguration;
     a.nst = nst;
     const int smem = Cfg::smem(nst, a.res_bytes);
-    cudaError_t e = cudaFuncSetAttribute(k_conv_fwd_gen<BN, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem<k_conv_fwd_gen<BN, RES>>(smem);
     if (e != cudaSuccess) return e;
     const int ntiles = a.n_row * a.n_col;
     const int grid = ntiles < conv_num_sms() ? ntiles : conv_num_sms();
@@ -1941,7 +1941,7 @@ static cudaError_t launch_dw_gen_bn(const uint2 *rec, const CUtensorMap &mD, Con
     if (Cfg::smem(nst, a.groups, kpos) > GEN_SMEM_MAX) return cudaErrorInvalidConfiguration;
     a.nst = nst;
     const int smem = Cfg::smem(nst, a.groups, kpos);
-    cudaError_t e = cudaFuncSetAttribute(k_conv_dw_gen<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem<k_conv_dw_gen<BN>>(smem);
     if (e != cudaSuccess) return e;
     const int ntiles = a.n_row * a.n_col * a.n_split;
     const int grid = ntiles < conv_num_sms() ? ntiles : conv_num_sms();
@@ -1953,8 +1953,7 @@ template <int BN, bool ROWBOX, bool RES, bool FWD>
 static cudaError_t launch_tap_bn(const CUtensorMap &mA, const CUtensorMap &mB, const CUtensorMap &mR, ConvGemmArgs a,
                                  DsPlan pl, cudaStream_t st) {
     const int smem = pl.nst * pl.stage + pl.res_bytes + pl.epi_bytes + 1024 + 256;
-    cudaError_t e = cudaFuncSetAttribute(k_conv_tap_gemm<BN, ROWBOX, RES, FWD>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem<k_conv_tap_gemm<BN, ROWBOX, RES, FWD>>(smem);
     if (e != cudaSuccess) return e;
     const int ntiles = a.n_row * a.n_col;
     const int grid = ntiles < conv_num_sms() ? ntiles : conv_num_sms();
@@ -2005,7 +2004,7 @@ cudaError_t launch_dwhat_pmc(const float *t_out, const int *q, const float *s, c
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     if (bulk) {
-        cudaError_t e = cudaFuncSetAttribute(k_dwhat_pmc<NPT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = allow_smem<k_dwhat_pmc<NPT, true>>(smem);
         if (e != cudaSuccess) return e;
         k_dwhat_pmc<NPT, true><<<(unsigned)blocks, 256, smem, st>>>(t_out, q, s, vdot, g_up, P, C, c, D, count);
     } else {
@@ -2287,7 +2286,7 @@ cudaError_t launch_conv_dw_tma(const ConvGeom &g, int ni, int C_out, const LifCo
     const int grid = ntiles < conv_num_sms() ? ntiles : conv_num_sms();
 #define DSTD_DWT(BNV)                                                                                            \
     {                                                                                                            \
-        cudaError_t e = cudaFuncSetAttribute(k_conv_dw_tma<BNV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); \
+        cudaError_t e = allow_smem<k_conv_dw_tma<BNV>>(smem);                                                    \
         if (e != cudaSuccess) return e;                                                                          \
         k_conv_dw_tma<BNV><<<grid, DWT_THREADS, smem, st>>>(mS, mD, a);                                         \
         return cudaGetLastError();                                                                               \
@@ -2313,7 +2312,7 @@ cudaError_t launch_bin_S(const float *t, long long P, int C, int Ct, const LifCo
     const int R = C >= BINS_THREADS ? 1 : BINS_THREADS / C;
     const int smem = 2 * R * Mp * C * 2;
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_bin_S, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem<k_bin_S>(smem);
     if (e != cudaSuccess) return e;
     const long long ngroups = (P + R - 1) / R;
     int per_sm = (227 * 1024) / smem;

@@ -130,19 +130,15 @@ cudaError_t launch_exact_fwd(const float *t_in, const float *W, int B, int N_in,
                                         N_out, nullptr, st);
     if (e != cudaSuccess) return e;
     const size_t smem_sort = (size_t)P * 8;
-    if (smem_sort > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_exact_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sort);
-        if (e != cudaSuccess) return e;
-    }
+    e = allow_smem<k_exact_sort>((long long)smem_sort);
+    if (e != cudaSuccess) return e;
     k_exact_sort<<<B, EXACT_SORT_THREADS, smem_sort, st>>>(t_in, N_in, c, t_end, P, ws.perm, ws.t_start, ws.iv,
                                                           ws.count);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t smem_walk = (size_t)N_in * (sizeof(float4) + 8);
-    if (smem_walk > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_exact_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_walk);
-        if (e != cudaSuccess) return e;
-    }
+    e = allow_smem<k_exact_walk>((long long)smem_walk);
+    if (e != cudaSuccess) return e;
     dim3 grid((N_out + EXACT_WALK_THREADS - 1) / EXACT_WALK_THREADS, B);
     k_exact_walk<<<grid, EXACT_WALK_THREADS, smem_walk, st>>>(ws.Wt, N_in, N_out, c, kmax, ws.perm, ws.t_start,
                                                              ws.iv, ws.count, t_out);
@@ -257,10 +253,8 @@ cudaError_t launch_exact_bwd(const float *t_in, const float *W, const float *t_o
                                         N_out, nullptr, st);
     if (e != cudaSuccess) return e;
     const size_t smem = (size_t)N_in * sizeof(float);
-    if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_exact_slope, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    e = allow_smem<k_exact_slope>((long long)smem);
+    if (e != cudaSuccess) return e;
     k_exact_slope<<<dim3((N_out + EXACT_BWD_THREADS - 1) / EXACT_BWD_THREADS, B), EXACT_BWD_THREADS, smem, st>>>(
         t_in, ws.Wt, t_out, g_out, N_in, N_out, c, ws.coef);
     e = cudaGetLastError();

@@ -7,6 +7,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/dstd.h"
 
 namespace dstd {
@@ -448,6 +450,28 @@ __device__ __forceinline__ void finish_neuron(const LifConst &c, const ScanState
 constexpr unsigned int STATUS_TIMEOUT = 1u;
 cudaError_t status_read(unsigned int *out, int clear);
 cudaError_t launch_wait_selftest(unsigned long long limit_ns, cudaStream_t st);
+
+// Lets a kernel launch with `bytes` of dynamic shared memory. The limit is one
+// number per kernel, shared by every thread that launches it: it is only ever
+// set to the most that the kernel can have, so that no thread lowers it between
+// another's call and launch (which would be refused).
+template <auto Kernel>
+cudaError_t allow_smem(long long bytes) {
+    static std::atomic<int> most{0};
+    int limit = most.load(std::memory_order_relaxed);
+    if (limit == 0) {
+        int dev = 0, optin = 0;
+        cudaFuncAttributes a;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, Kernel);
+        if (e != cudaSuccess) return e;
+        limit = optin - (int)a.sharedSizeBytes;
+        most.store(limit, std::memory_order_relaxed);
+    }
+    if (bytes > limit) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+}
 
 // ---------------------------------------------------------------------------
 // Kernel launch entry points (host functions that launch on a stream).

@@ -1232,7 +1232,7 @@ cudaError_t launch_narrow_fwd(const float *t, const float *W, int B, int N_in, i
     if (smem > kNarrowMaxSmem) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
 #define DSTD_NARROW_FWD(S, NO)                                                                                    \
-    e = cudaFuncSetAttribute(k_narrow_fwd<S, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
+    e = allow_smem<k_narrow_fwd<S, NO>>((long long)smem);                                                         \
     if (e != cudaSuccess) return e;                                                                                \
     k_narrow_fwd<S, NO><<<B, NARROW_FWD_THREADS, smem, st>>>(t, W, N_in, N_out, c, t_out, q, s, vdot, penalty, ce);
 #define DSTD_NARROW_FWD_NO(S) \
