@@ -706,23 +706,24 @@ def _padded_m(M):
 
 def conv_step_units(n):
     """Algorithmic work of one training step of a conv network, per kernel
-    kind (SURVEY 8(d) units, summed over the layers):
+    kind, summed over the layers:
       contractions  4 x positions x k^2 C_in x C_out flops each (two grid
                     weights per input spike), with the dense tensor-core
                     flops of the binned formulation beside them;
       binning       read the input spike times (4 B), write the binned
                     operand in the NHWC + grid-step layout (M x 2 B each),
-                    or, for layers whose contraction generates it on chip
-                    (the library's rules for the forward of large 64 -> 64
-                    layers and for dW of 3x3 layers with 64 outputs), an
+                    or, where the layer's contraction generates it on chip, an
                     8-byte record;
-      scan/solve    read w^ (positions x M_p x C_out x 4 B), write 16 B per neuron;
+      scan/solve    read w^ (positions x M_p x C_out x 4 B), write 16 B per
+                    neuron, where it does not run inside the contraction;
       dw^           read 20 B per neuron, write positions x M_p x C_out x 2 B;
       weight prep   read W (4 B), write its bf16 copy (forward and, where the
                     input gradient is needed, the transposed one);
       AdamW         28 B per weight.
     The dense readout counts as a dense layer (its own kinds on the
-    few-output path). Returns (flops, dense_flops, bytes) dicts."""
+    few-output path). Which form a conv layer takes is asked of the library.
+    Returns (flops, dense_flops, bytes) dicts."""
+    from paper_2607_14672_gb300 import dstd
     from paper_2607_14672_gb300.net import narrow_layer
     algo_f, dense_f, algo_b = {}, {}, {}
 
@@ -743,12 +744,12 @@ def conv_step_units(n):
             for kk in kinds:
                 add(algo_f, kk, f)
                 add(dense_f, kk, df)
-            on_chip = n.math == "bf16" and O == 64 and st == 1 and Mp in (32, 64)
-            rec_fwd = on_chip and C <= 64 and k > 1 and P >= 300 * 152
-            rec_bwd = on_chip and k == 3
+            route = dstd.conv_route(B, H, Wd, C, O, k, st, pad, n.p[l], n.math)
+            rec_fwd, rec_bwd = ("implicit" in route and x not in route for x in ("fwd_binned", "dw_binned"))
             add(algo_b, "binning", Pin * 4 + Pin * (8 if rec_fwd else M * 2))
             add(algo_b, "binning_T", Pin * 4 + Pin * (8 if rec_bwd else M * 2))
-            add(algo_b, "scan_solve", P * O * Mp * 4 + P * O * 16)
+            if "fused_scan" not in route:
+                add(algo_b, "scan_solve", P * O * Mp * 4 + P * O * 16)
             add(algo_b, "dwhat", P * O * 20 + P * O * Mp * 2)
             add(algo_b, "prep_weights", (O * K * 6) * (2 if l > 0 else 1))
             add(algo_b, "adamw", 28 * O * K)
