@@ -1,18 +1,19 @@
 // Conv contractions on sm_103a that take each part of their source image once:
 // forward and dS by rows (tcgen05, bf16 operands, fp32 accumulation).
 //
-// A work item is a run of output rows of one image, one tile of output
-// positions wide (ppt = 128 / Mp positions per 128-row MMA tile, NT tiles) and
-// BN channels deep. The item walks the source rows that its output rows read;
-// the box of one source row (positions x grid steps x 64 channels, bf16, in
-// shared memory) feeds every filter row and column that reads it, so up to
-// ceil(k / stride) (forward) or k (dS) output rows are in flight, each in its
-// own TMEM accumulator. The one-row-at-a-time kernels load a box per filter
+// A work item is a run of output rows of one image, NT tiles of output
+// positions wide (ppt = 128 / Mp positions per 128-row MMA tile) and 64 channels
+// deep: the forward of 64 -> 64 layers at stride 1 (one tile), dS of layers with
+// 64 input channels (any number of output channels, strides 1 and 2). The item
+// walks the source rows that its output rows read; the box of one source row
+// (positions x grid steps x 64 channels, bf16, in shared memory) feeds every
+// filter row and column that reads it, so up to k output rows are in flight,
+// each in its own TMEM accumulator. The one-row-at-a-time kernels load a box per filter
 // row and keep two in flight, 12 to 24 MMAs per load of about 1.4 us; here a
 // box serves 36 to 72 MMAs. What bounds this kernel then: dS at 64 channels
 // runs at 53 clocks per N = 64 MMA, of which reading the operands from shared
 // memory takes 48 (64 -> 64 at 28 x 28, B = 256, M = 64: 1.35 -> 0.68 ms); the
-// forward is bound by the scan's instructions (the same layer: 2.38 -> 1.75 ms
+// forward is bound by the scan's instructions (the same layer: 2.38 -> 1.66 ms
 // with the binning).
 //
 //   forward  the box holds the binned input and is generated on chip from 8
@@ -58,19 +59,20 @@ constexpr int MAX_NSTA = 4;    // stages of source boxes
 constexpr int MAX_NSTB = 8;    // stages of filter slices
 constexpr int GEN_WARPS = 4;   // forward: generator warps
 constexpr int MMA_WARPS = 4;   // issuing warps: output row n by warp n mod 4
-constexpr int GEN_SLOTS = 7;   // (position, channel) slots of a generator thread per box, at most
+constexpr int GEN_SLOTS = 5;   // (position, channel) slots of a generator thread per box, at most (7x7, 32 grid steps)
+constexpr int ROWS_BN = 64;    // output channels of a tile
 constexpr int EPI_LDF = 36;    // forward epilogue: floats per neuron row of 32 grid steps (read as float4)
 constexpr int EPI_LDG = 33;    // dS epilogue: floats per grid-step row of 32 channels
 constexpr int SILENT = -128;   // grid step of a record, and kept step of a slot, without a spike
 
 struct RowsPlan {
-    int n_items, n_xt, n_col, n_strip, R;  // items; position tiles, column tiles, strips of R output rows
+    int n_items, n_xt, n_col, n_strip, R;  // items; position tiles, dS: column tiles (of 64 channels), strips of R output rows
     int gh, gw, sh, sw;                    // output and source grids
-    int s, k, pad, ncb, cb_inner;
+    int s, k, pad, ncb, cb_inner;          // forward: s = 1, ncb = 1
     int Mp, ppt;
-    int nsta, nstb, npos, slots;           // stages; positions of a box, and places they take (planes by x mod s)
+    int nsta, nstb, npos;                  // stages; positions of a box
     int kwg;                               // filter columns per streamed stage (k or 1)
-    int box_bytes, stage_bytes, res_bytes; // res_bytes > 0: all filter slices of the column tile stay resident
+    int box_bytes, stage_bytes, res_bytes; // res_bytes > 0: all filter slices stay resident
     int nset;                              // epilogue warps / 4
     int xs_mul, xs_add;                    // first source position of tile xt: xt xs_mul + xs_add
     int off_b, off_epi, off_state, off_kept, off_bar, smem;  // shared-memory layout (from a 1 KB boundary), and its size
@@ -82,7 +84,6 @@ struct RowsArgs {
     const uint2 *rec;   // forward: the source's records (k_bin_rec), C_t channels
     const float *t_in;  // dS: the layer input's spike times, C_t channels
     int C_t;
-    int C_out;          // channels of the output grid (forward: C_out; dS: C_in padded)
     float *t_out;       // forward
     int *q_out;
     float *s_out, *vdot_out;
@@ -110,10 +111,12 @@ __device__ __forceinline__ uint32_t rows_sw128(int r, int c) {
 // (the order in which an output row's filter rows come up).
 template <bool FWD>
 struct Item {
-    int b, xt, ct, ya, yb, sr, sr_end;  // sr steps by +-1 up to and including sr_end
+    int b, xt, ct, ya, yb, sr, sr_end;  // (ct: dS only) sr steps by +-1 up to and including sr_end
     __device__ __forceinline__ void decode(const RowsPlan &p, int it) {
-        ct = it % p.n_col;
-        it /= p.n_col;
+        if (!FWD) {  // rows_pick takes one column tile; but dS without the index came out 2 to 3% slower
+            ct = it % p.n_col;
+            it /= p.n_col;
+        }
         xt = it % p.n_xt;
         it /= p.n_xt;
         const int strip = it % p.n_strip;
@@ -121,9 +124,9 @@ struct Item {
         ya = strip * p.R;
         yb = ya + p.R < p.gh ? ya + p.R : p.gh;
         if (FWD) {
-            sr = ya * p.s - p.pad;
+            sr = ya - p.pad;
             if (sr < 0) sr = 0;
-            sr_end = (yb - 1) * p.s - p.pad + p.k - 1;
+            sr_end = yb - 1 - p.pad + p.k - 1;
             if (sr_end > p.sh - 1) sr_end = p.sh - 1;
         } else {
             sr = (yb - 1 + p.pad) >> (p.s - 1);  // strides are 1 or 2
@@ -136,24 +139,14 @@ struct Item {
     __device__ __forceinline__ bool done(int r) const { return FWD ? r > sr_end : r < sr_end; }
     // output row that source row r reaches through filter row kh, or -1
     __device__ __forceinline__ int out_row(const RowsPlan &p, int r, int kh) const {
-        int y;
-        if (FWD) {
-            y = r + p.pad - kh;
-            if (y < 0) return -1;
-            if (p.s == 2) {
-                if (y & 1) return -1;
-                y >>= 1;
-            }
-        } else {
-            y = r * p.s - p.pad + kh;
-        }
+        const int y = FWD ? r + p.pad - kh : r * p.s - p.pad + kh;
         return y >= ya && y < yb ? y : -1;
     }
     __device__ __forceinline__ int seq(int y) const { return FWD ? y - ya : yb - 1 - y; }
     // whether source row r is the first / the last that output row y reads
     __device__ __forceinline__ bool first_of(const RowsPlan &p, int r, int y) const {
         if (FWD) {
-            const int f = y * p.s - p.pad;
+            const int f = y - p.pad;
             return r == (f < 0 ? 0 : f);
         }
         const int f = (y + p.pad) >> (p.s - 1);
@@ -161,7 +154,7 @@ struct Item {
     }
     __device__ __forceinline__ bool last_of(const RowsPlan &p, int r, int y) const {
         if (FWD) {
-            const int l = y * p.s - p.pad + p.k - 1;
+            const int l = y - p.pad + p.k - 1;
             return r == (l > p.sh - 1 ? p.sh - 1 : l);
         }
         const int l = y + p.pad - (p.k - 1);
@@ -319,12 +312,12 @@ __device__ __forceinline__ bool walk_rolled(unsigned lanes, const LifConst &c, c
 // on waits, addresses and commits, which the other warps' MMAs now cover (one
 // warp: 82 to 130 clocks per N = 64 MMA over the whole loop, of which the
 // tensor core needs 48).
-template <int BN, int NT, bool FWD>
+template <int NT, bool FWD>
 struct Roles {
     static constexpr int W_B = FWD ? GEN_WARPS : 1;  // the filter warp
     static constexpr int W_MMA = W_B + 1;
     static constexpr int W_EPI = W_MMA + MMA_WARPS;
-    static constexpr int SLOT_COLS = NT * BN;
+    static constexpr int SLOT_COLS = NT * ROWS_BN;
     static constexpr int NA = 512 / SLOT_COLS > 8 ? 8 : 512 / SLOT_COLS;  // accumulators (output rows)
     static constexpr int CH = SLOT_COLS / 32;                            // 32-channel chunks of an output row
     static __host__ __device__ constexpr int threads(int nset) { return (W_EPI + 4 * nset) * 32; }
@@ -333,15 +326,16 @@ constexpr int FWD_MAX_THREADS = (GEN_WARPS + 1 + MMA_WARPS + 16) * 32;
 constexpr int DS_MAX_THREADS = (2 + MMA_WARPS + 8) * 32;
 
 // SLOTS: (position, channel) slots of a generator thread per box (forward)
-template <int BN, int NT, bool FWD, int SLOTS>
+template <int NT, bool FWD, int SLOTS>
 __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
     k_conv_rows(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const __grid_constant__ RowsArgs a, const __grid_constant__ RowsPlan p) {
-    using Ro = Roles<BN, NT, FWD>;
+    using Ro = Roles<NT, FWD>;
+    static_assert(!FWD || NT == 1, "the forward takes one position tile");
     constexpr int NA = Ro::NA, CH = Ro::CH;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    constexpr int SLICE = BN * 128;  // one filter slice: BN channels x 64 of K
+    constexpr int SLICE = ROWS_BN * 128;  // one filter slice: ROWS_BN channels x 64 of K
     uint8_t *bbuf = smem + p.off_b;  // resident filters, or the ring of slices
     float *epi = reinterpret_cast<float *>(smem + p.off_epi);
     float4 *state = reinterpret_cast<float4 *>(smem + p.off_state);
@@ -356,8 +350,9 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(res_full + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int Mp = p.Mp, k = p.k, ncb = p.ncb;
-    const int cbo_n = p.cb_inner ? 1 : ncb, cbi_n = p.cb_inner ? ncb : 1;  // boxes outside / inside the filter columns
+    const int Mp = p.Mp, k = p.k, ncb = p.ncb;  // forward: one channel block (as constants 3% slower)
+    const bool cb_inner = p.cb_inner != 0;
+    const int cbo_n = cb_inner ? 1 : ncb, cbi_n = cb_inner ? ncb : 1;  // boxes outside / inside the filter columns
     const int kc = ncb * 64;
 
     if (threadIdx.x == 0) {
@@ -397,31 +392,27 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
         // the generators 3600 clocks per box.)
         const int g0 = threadIdx.x >> 6, c = threadIdx.x & 63;
         Item<FWD> nx;
-        int n_it = blockIdx.x, n_sr = 0, n_cb = 0;
+        int n_it = blockIdx.x, n_sr = 0;
         if (n_it < p.n_items) {
             nx.decode(p, n_it);
             n_sr = nx.sr;
         }
         uint2 tn[SLOTS];
         auto load_next = [&]() {
-            const int ch = n_cb * 64 + c;
-            const bool on = n_it < p.n_items && ch < a.C_t;
+            const bool on = n_it < p.n_items && c < a.C_t;
             const int x0 = on ? nx.xt * p.xs_mul + p.xs_add : 0;
-            const uint2 *src = on ? a.rec + (((long long)nx.b * p.sh + n_sr) * p.sw + x0) * a.C_t + ch : nullptr;
+            const uint2 *src = on ? a.rec + (((long long)nx.b * p.sh + n_sr) * p.sw + x0) * a.C_t + c : nullptr;
 #pragma unroll
             for (int u = 0; u < SLOTS; ++u) {
                 const int i = g0 + 2 * u;
                 tn[u] = make_uint2((uint32_t)SILENT, 0u);
                 if (on && i < p.npos && x0 + i >= 0 && x0 + i < p.sw) tn[u] = __ldg(src + (long long)i * a.C_t);
             }
-            if (n_it < p.n_items && ++n_cb == ncb) {
-                n_cb = 0;
-                if (nx.done(++n_sr)) {
-                    n_it += gridDim.x;
-                    if (n_it < p.n_items) {
-                        nx.decode(p, n_it);
-                        n_sr = nx.sr;
-                    }
+            if (n_it < p.n_items && nx.done(++n_sr)) {
+                n_it += gridDim.x;
+                if (n_it < p.n_items) {
+                    nx.decode(p, n_it);
+                    n_sr = nx.sr;
                 }
             }
         };
@@ -429,55 +420,46 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
         int sa = 0;
         uint32_t ph = 0;
         bool ok = true;
-        const int planes = p.s, per_plane = p.slots / p.s;
         for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x) {
             Item<FWD> w;
             w.decode(p, it);
-            for (int sr = w.sr; !w.done(sr) && ok; ++sr) {
-                for (int cbo = 0; cbo < cbo_n; ++cbo) {
-                    for (int cbi = 0; cbi < cbi_n; ++cbi) {
-                        uint2 cur[SLOTS];
+            for (int sr = w.sr; !w.done(sr); ++sr) {
+                uint2 cur[SLOTS];
 #pragma unroll
-                        for (int u = 0; u < SLOTS; ++u) cur[u] = tn[u];
-                        load_next();
-                        if (cbi == 0) {  // the stage's previous MMAs are done with it
-                            int got = 1;
-                            if (lane == 0) got = tc::mbar_wait_spin(&empty_a[sa], ph ^ 1u) ? 1 : 0;
-                            if (!__shfl_sync(0xffffffffu, got, 0)) {
-                                if (lane == 0) rows_set_status(STATUS_TIMEOUT);
-                                ok = false;
-                                break;
-                            }
-                        }
-                        const uint32_t box = tc::smem_u32(smem + sa * p.stage_bytes + cbi * p.box_bytes);
-                        int8_t *kp = kept + ((sa * cbi_n + cbi) * p.npos) * 64 + c;
+                for (int u = 0; u < SLOTS; ++u) cur[u] = tn[u];
+                load_next();
+                int got = 1;  // the stage's previous MMAs are done with it
+                if (lane == 0) got = tc::mbar_wait_spin(&empty_a[sa], ph ^ 1u) ? 1 : 0;
+                if (!__shfl_sync(0xffffffffu, got, 0)) {
+                    if (lane == 0) rows_set_status(STATUS_TIMEOUT);
+                    ok = false;
+                    break;
+                }
+                const uint32_t box = tc::smem_u32(smem + sa * p.stage_bytes);
+                int8_t *kp = kept + sa * p.npos * 64 + c;
 #pragma unroll
-                        for (int u = 0; u < SLOTS; ++u) {
-                            const int i = g0 + 2 * u;
-                            if (i >= p.npos) break;
-                            const int kk = (int)cur[u].x;
-                            const uint32_t wq = cur[u].y;
-                            const int place = planes == 1 ? i : (i & 1) * per_plane + (i >> 1);
-                            const int row0 = place * Mp, old = kp[i * 64];
-                            if (old != SILENT) {
-                                if (old >= 0) rows_sts_u16(box + rows_sw128(row0 + old, c), 0);
-                                if (old + 1 < a.c.M) rows_sts_u16(box + rows_sw128(row0 + old + 1, c), 0);
-                            }
-                            if (kk != SILENT) {
-                                if (kk >= 0) rows_sts_u16(box + rows_sw128(row0 + kk, c), (uint16_t)(wq & 0xffffu));
-                                if (kk + 1 < a.c.M) rows_sts_u16(box + rows_sw128(row0 + kk + 1, c), (uint16_t)(wq >> 16));
-                            }
-                            if (kk != old) kp[i * 64] = (int8_t)kk;
-                        }
+                for (int u = 0; u < SLOTS; ++u) {
+                    const int i = g0 + 2 * u;
+                    if (i >= p.npos) break;
+                    const int kk = (int)cur[u].x;
+                    const uint32_t wq = cur[u].y;
+                    const int row0 = i * Mp, old = kp[i * 64];
+                    if (old != SILENT) {
+                        if (old >= 0) rows_sts_u16(box + rows_sw128(row0 + old, c), 0);
+                        if (old + 1 < a.c.M) rows_sts_u16(box + rows_sw128(row0 + old + 1, c), 0);
                     }
-                    if (!ok) break;
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(&full_a[sa]);
-                    if (++sa == p.nsta) {
-                        sa = 0;
-                        ph ^= 1u;
+                    if (kk != SILENT) {
+                        if (kk >= 0) rows_sts_u16(box + rows_sw128(row0 + kk, c), (uint16_t)(wq & 0xffffu));
+                        if (kk + 1 < a.c.M) rows_sts_u16(box + rows_sw128(row0 + kk + 1, c), (uint16_t)(wq >> 16));
                     }
+                    if (kk != old) kp[i * 64] = (int8_t)kk;
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&full_a[sa]);
+                if (++sa == p.nsta) {
+                    sa = 0;
+                    ph ^= 1u;
                 }
             }
         }
@@ -514,7 +496,7 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
         __syncwarp();
     } else if (warp == Ro::W_B) {
         const uint32_t lead = tc::elect_one();
-        if (p.res_bytes) {  // every slice of the single column tile, once
+        if (p.res_bytes) {  // every slice, once
             const int n = k * k * ncb;
             tc::mbar_expect_tx_if(lead, res_full, (uint32_t)(n * SLICE));
             for (int q = 0; q < n; ++q) {
@@ -544,7 +526,7 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                                 for (int kw = kw0; kw < kw0 + p.kwg; ++kw)
                                     for (int cbi = 0; cbi < cbi_n; ++cbi, dst += SLICE)
                                         tc::tma_load_2d_if(lead, dst, &mapB, &full_b[sb],
-                                                           (kh * k + kw) * kc + (cbo + cbi) * 64, w.ct * BN);
+                                                           (kh * k + kw) * kc + (cbo + cbi) * 64, FWD ? 0 : w.ct * ROWS_BN);
                                 if (++sb == p.nstb) {
                                     sb = 0;
                                     ph ^= 1u;
@@ -559,7 +541,7 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
         __syncwarp();
     } else if (warp >= Ro::W_MMA && warp < Ro::W_EPI) {
         const uint32_t mw = (uint32_t)(warp - Ro::W_MMA);
-        constexpr uint32_t idesc = idesc_kk(BN);
+        constexpr uint32_t idesc = idesc_kk(ROWS_BN);
         const uint32_t lead = tc::elect_one();
         const bool res = p.res_bytes != 0;
         int sa = 0, sb = 0;
@@ -567,7 +549,7 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
         uint32_t n0 = 0;  // output rows of the items before
         // low descriptor words; slices of one channel block are ncb apart when resident
         const uint32_t res_lo = tc::sdesc_kk_lo(tc::smem_u32(bbuf));
-        const uint32_t b_step = (uint32_t)((res && !p.cb_inner ? ncb : 1) * (SLICE >> 4));
+        const uint32_t b_step = (uint32_t)((res && !cb_inner ? ncb : 1) * (SLICE >> 4));
         const bool three = k == 3 && p.kwg == 3 && cbi_n == 1;
         const uint32_t tmem_u = tc::uniform(tmem);
         bool ok = !res || tc::mbar_wait_warp(res_full, 0);
@@ -631,10 +613,10 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                                     if (NT == 2 && o < 0) continue;
                                     const uint32_t alo = st + (uint32_t)(cbi * (p.box_bytes >> 4) + o);
                                     const uint32_t on = !(fresh && kw == p.kfirst[t] && cbi == 0);  // adds to the tile
-                                    tc::mma_kk(acc + t * BN, alo, bo, idesc, on);
+                                    tc::mma_kk(acc + t * ROWS_BN, alo, bo, idesc, on);
 #pragma unroll
                                     for (int kk = 1; kk < 4; ++kk)
-                                        tc::mma_kk(acc + t * BN, alo + 2 * kk, bo + 2 * kk, idesc, 1u);
+                                        tc::mma_kk(acc + t * ROWS_BN, alo + 2 * kk, bo + 2 * kk, idesc, 1u);
                                 }
                             };
                             if (lead && mine) {
@@ -749,9 +731,9 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                 }
                 __syncwarp();
             }
-            const int x = (w.xt * NT + c / (BN / 32)) * p.ppt + pp;
+            const int x = w.xt * p.ppt + pp;
             const bool on = more && x < p.gw && !fail;
-            const int pos = (w.b * p.gh + w.ya + r) * p.gw + x, ch = w.ct * BN + (c % (BN / 32)) * 32 + lane;
+            const int pos = (w.b * p.gh + w.ya + r) * p.gw + x, ch = c * 32 + lane;
             // the state the walk starts from (upper: the lower quarter's end), then the spike's bin or the end
             // state: (q, v0, I0, hi) or (-1, v, I, -)
             float4 h = make_float4(__int_as_float(-1), 0.f, 0.f, 0.f);
@@ -800,7 +782,7 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                     st.hi = h.w;
                 }
                 scan_finish(a.c, st);
-                finish_neuron(a.c, st, f_pos, f_ch, a.C_out, a.rowsum, a.t_out, a.q_out, a.s_out, a.vdot_out, pacc);
+                finish_neuron(a.c, st, f_pos, f_ch, ROWS_BN, a.rowsum, a.t_out, a.q_out, a.s_out, a.vdot_out, pacc);
             }
             __syncwarp();
         }
@@ -814,13 +796,13 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
         }
     } else {
         // dS: with two tiles per row, group g takes tile g; with one, every
-        // other row. A warp reads its lane quarter of all BN columns; lane u of
+        // other row. A warp reads its lane quarter of all ROWS_BN columns; lane u of
         // a chunk then owns input channel u and picks its two grid steps.
         const int ew = warp - Ro::W_EPI, group = ew >> 2, quarter = warp & 3;
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         float *tb = epi + ew * 32 * EPI_LDG;
         const int pp = (quarter * 32) / Mp, m_base = (quarter * 32) % Mp;
-        constexpr int NCH = BN / 32;
+        constexpr int NCH = ROWS_BN / 32;
         uint32_t n = 0;
         bool ok = true;
         for (int it = blockIdx.x; it < p.n_items && ok; it += gridDim.x) {
@@ -839,7 +821,7 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                 float ti[NCH];
 #pragma unroll
                 for (int h = 0; h < NCH; ++h) {
-                    const int col = w.ct * BN + h * 32 + lane;
+                    const int col = w.ct * ROWS_BN + h * 32 + lane;
                     ti[h] = x < p.gw && col < a.C_t ? __ldg(a.t_in + pos * a.C_t + col) : INFINITY;
                 }
                 if (__any_sync(0xffffffffu, !tc::mbar_wait_sleep(&acc_full[slot], (n / NA) & 1u))) {
@@ -847,7 +829,7 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                     break;
                 }
                 tc::tc_fence_after();
-                const uint32_t acc = tmem + lane_base + slot * Ro::SLOT_COLS + tau * BN;
+                const uint32_t acc = tmem + lane_base + slot * Ro::SLOT_COLS + tau * ROWS_BN;
 #pragma unroll 1
                 for (int h = 0; h < NCH; ++h) {
                     {
@@ -872,7 +854,7 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
                             float g = 0.f;
                             if (k0 >= 0) g = fmaf(tb[k0 * EPI_LDG + lane], bw.dR, g);
                             if (k0 + 1 < 32 && kb + 1 < a.c.M) g = fmaf(tb[(k0 + 1) * EPI_LDG + lane], bw.dL, g);
-                            if (g != 0.f) atomicAdd(a.g_t_in + pos * a.C_t + w.ct * BN + h * 32 + lane, g);
+                            if (g != 0.f) atomicAdd(a.g_t_in + pos * a.C_t + w.ct * ROWS_BN + h * 32 + lane, g);
                         }
                     }
                     __syncwarp();
@@ -1275,7 +1257,8 @@ constexpr int BAR_BYTES = (2 * MAX_NSTA + 2 * MAX_NSTB + 16 + 1) * 8 + 8;  // ba
 // Behind the source boxes: filters, epilogue rows (32 x 32 values a warp),
 // forward: the lower quarters' states (64 grid steps) and the kept grid steps
 // of the generator slots; the barriers last
-bool rows_layout(bool fwd, RowsPlan &p, int slice) {
+bool rows_layout(bool fwd, RowsPlan &p) {
+    constexpr int slice = ROWS_BN * 128;
     const int cbi = p.cb_inner ? p.ncb : 1;
     const long long b = p.res_bytes ? (long long)p.res_bytes : (long long)p.nstb * p.kwg * cbi * slice;
     const long long off_epi = (long long)p.nsta * p.stage_bytes + b;
@@ -1316,8 +1299,7 @@ void rows_strips(RowsPlan &p, int ni) {
 // one-row-at-a-time kernels: strides above 2, filters wider than their
 // padding allows (an output row without a source row), more output rows in
 // flight than accumulators, or too little shared memory.
-bool rows_plan(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner, int BN, int NT, int nset,
-               RowsPlan &p) {
+bool rows_plan(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner, int NT, int nset, RowsPlan &p) {
     p = RowsPlan{};
     p.s = g.s;
     p.k = g.k;
@@ -1328,27 +1310,22 @@ bool rows_plan(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_i
     p.gw = fwd ? g.Wo : g.W;
     p.sh = fwd ? g.H : g.Ho;
     p.sw = fwd ? g.W : g.Wo;
-    p.ncb = (fwd ? g.C : C_out) / 64;
+    p.ncb = fwd ? 1 : C_out / 64;
     p.cb_inner = cb_inner && p.ncb > 1;
     p.nset = nset;
-    const int cols = fwd ? C_out : g.C;
-    p.n_col = cols / BN;
-    if (g.s > 2 || g.k > MAX_K || g.k < g.s || g.p > g.k - 1 || cols % BN != 0) return false;
+    p.n_col = fwd ? 1 : g.C / ROWS_BN;
+    if (g.s > 2 || g.k > MAX_K || g.k < g.s || g.p > g.k - 1) return false;
     for (int t = 0; t < 2; ++t)
         for (int kw = 0; kw < MAX_K; ++kw) p.aoff[t][kw] = -1;
     if (fwd) {
-        p.n_xt = (p.gw + NT * p.ppt - 1) / (NT * p.ppt);
-        p.npos = p.s * (NT * p.ppt - 1) + p.k;
-        const int per_plane = (p.npos + p.s - 1) / p.s;
-        p.slots = p.s * per_plane;
-        for (int t = 0; t < NT; ++t)
-            for (int kw = 0; kw < p.k; ++kw) p.aoff[t][kw] = (kw % p.s) * per_plane + kw / p.s + t * p.ppt;
-        p.xs_mul = NT * p.ppt * p.s;
+        p.n_xt = (p.gw + p.ppt - 1) / p.ppt;
+        p.npos = p.ppt - 1 + p.k;
+        for (int kw = 0; kw < p.k; ++kw) p.aoff[0][kw] = kw;
+        p.xs_mul = p.ppt;
         p.xs_add = -p.pad;
-        if ((p.npos + 1) / 2 > GEN_SLOTS) return false;
     } else if (p.s == 1) {
         p.n_xt = (p.gw + NT * p.ppt - 1) / (NT * p.ppt);
-        p.npos = p.slots = NT * p.ppt + p.k - 1;
+        p.npos = NT * p.ppt + p.k - 1;
         for (int t = 0; t < NT; ++t)
             for (int kw = 0; kw < p.k; ++kw) p.aoff[t][kw] = t * p.ppt + p.k - 1 - kw;
         p.xs_mul = NT * p.ppt;
@@ -1367,13 +1344,13 @@ bool rows_plan(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_i
             }
         for (int t = 0; t < 2; ++t)
             for (int kw = (t + p.pad) % 2; kw < p.k; kw += 2) p.aoff[t][kw] = (t + p.pad - kw) / 2 - lo;
-        p.npos = p.slots = p.ppt + hi - lo;
+        p.npos = p.ppt + hi - lo;
         p.xs_mul = p.ppt;
         p.xs_add = lo;
     }
     // output rows in flight at one source row, and one for the epilogue
-    const int flight = (fwd ? (p.k + p.s - 1) / p.s : p.k) + 1;
-    int NA = 512 / (NT * BN);
+    const int flight = p.k + 1;
+    int NA = 512 / (NT * ROWS_BN);
     if (NA > 8) NA = 8;
     if (flight > NA) return false;
     // every output row reads at least one source row
@@ -1382,7 +1359,7 @@ bool rows_plan(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_i
         for (int kh = 0; kh < p.k && !any; ++kh) {
             int r;
             if (fwd) {
-                r = y * p.s - p.pad + kh;
+                r = y - p.pad + kh;
             } else {
                 if ((y + p.pad - kh) < 0 || (y + p.pad - kh) % p.s != 0) continue;
                 r = (y + p.pad - kh) / p.s;
@@ -1399,22 +1376,21 @@ bool rows_plan(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_i
                 p.kfirst[t] = kw;
             }
     }
-    p.box_bytes = p.slots * Mp * 128;
+    p.box_bytes = p.npos * Mp * 128;
     p.stage_bytes = p.box_bytes * (p.cb_inner ? p.ncb : 1);
-    const int slice = BN * 128;
-    const long long res = (long long)p.k * p.k * p.ncb * slice;
+    const long long res = (long long)p.k * p.k * p.ncb * ROWS_BN * 128;
     p.nsta = 2;
     p.nstb = 0;
     p.kwg = p.k;
-    if (p.n_col == 1 && res < ROWS_SMEM_MAX) {
+    if (res < ROWS_SMEM_MAX) {
         p.res_bytes = (int)res;
-        if (!rows_layout(fwd, p, slice)) p.res_bytes = 0;
+        if (!rows_layout(fwd, p)) p.res_bytes = 0;
     }
     if (!p.res_bytes) {
         // as many stages of a whole filter row as fit, at least two; else of single filter columns
         for (int pass = 0; pass < 2; ++pass) {
             p.kwg = pass == 0 ? p.k : 1;
-            for (p.nstb = MAX_NSTB; p.nstb >= 2 && !rows_layout(fwd, p, slice);) --p.nstb;
+            for (p.nstb = MAX_NSTB; p.nstb >= 2 && !rows_layout(fwd, p);) --p.nstb;
             if (p.nstb >= 2) break;
         }
         if (p.nstb < 2) return false;
@@ -1422,40 +1398,25 @@ bool rows_plan(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_i
     while (!fwd && p.nsta < MAX_NSTA) {
         RowsPlan m = p;
         ++m.nsta;
-        if (!rows_layout(fwd, m, slice)) break;
+        if (!rows_layout(fwd, m)) break;
         p = m;
     }
     rows_strips(p, ni);
     return true;
 }
 
-template <int BN, int NT, bool FWD, int SLOTS>
-cudaError_t rows_launch_slots(const CUtensorMap &mA, const CUtensorMap &mB, const RowsArgs &a, const RowsPlan &p,
+template <int NT, bool FWD, int SLOTS>
+cudaError_t rows_launch(const CUtensorMap &mA, const CUtensorMap &mB, const RowsArgs &a, const RowsPlan &p,
                         cudaStream_t st) {
-    cudaError_t e = allow_smem<k_conv_rows<BN, NT, FWD, SLOTS>>(p.smem);
+    cudaError_t e = allow_smem<k_conv_rows<NT, FWD, SLOTS>>(p.smem);
     if (e != cudaSuccess) return e;
     const int grid = p.n_items < rows_num_sms() ? p.n_items : rows_num_sms();
-    k_conv_rows<BN, NT, FWD, SLOTS><<<grid, Roles<BN, NT, FWD>::threads(p.nset), p.smem, st>>>(mA, mB, a, p);
+    k_conv_rows<NT, FWD, SLOTS><<<grid, Roles<NT, FWD>::threads(p.nset), p.smem, st>>>(mA, mB, a, p);
     return cudaGetLastError();
 }
 
-// the generator's code is laid out for its slots (2 to 4 for 3x3 filters at either stride and 5x5 at 32 grid
-// steps): unrolled for the most there can be, it took 17 KB of the instruction cache
-template <int BN, int NT, bool FWD>
-cudaError_t rows_launch(const CUtensorMap &mA, const CUtensorMap &mB, const RowsArgs &a, const RowsPlan &p,
-                        cudaStream_t st) {
-    const int slots = FWD ? (p.npos + 1) / 2 : 1;
-    if constexpr (!FWD) {
-        return rows_launch_slots<BN, NT, FWD, 1>(mA, mB, a, p, st);
-    } else {
-        if (slots <= 2) return rows_launch_slots<BN, NT, FWD, 2>(mA, mB, a, p, st);
-        if (slots <= 3) return rows_launch_slots<BN, NT, FWD, 3>(mA, mB, a, p, st);
-        return rows_launch_slots<BN, NT, FWD, GEN_SLOTS>(mA, mB, a, p, st);
-    }
-}
-
 struct Tile {
-    int BN, NT, nset;
+    int NT, nset;
 };
 
 // The tile shapes to try, best first, where this kernel is the faster one.
@@ -1463,9 +1424,9 @@ struct Tile {
 // whole warps too), every layer shape of the 9- and 20-layer networks:
 //   forward  64 output channels of one channel block at stride 1: 1.01 to 1.07
 //            times faster from about 300 output positions per SM on (binning
-//            included), 0.86 to 0.96 below; two channel blocks 0.82, stride 2
-//            0.95 to 1.02, 1x1 0.91, 128 and more output channels (filters
-//            streamed): 0.6 to 0.9;
+//            included), 0.86 to 0.96 below. Not built: two channel blocks
+//            (0.82), stride 2 (0.95 to 1.02), 128 and more output channels
+//            (filters streamed, 0.6 to 0.9); 1x1 0.91;
 //   dS       64 input channels: 1.2 to 2.3 times faster (64 -> 64 at 28 x 28:
 //            1.55; 64 -> 128 at stride 2: 2.0), 0.87 to 1 on a few thousand
 //            positions; 128 input channels: 0.8 to 0.96, wider: 0.5 to 0.9.
@@ -1475,14 +1436,14 @@ bool rows_pick(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_i
     if (fwd) {
         if (C_out != 64 || g.C != 64 || g.s != 1 || g.k == 1) return false;
         if ((long long)ni * g.Ho * g.Wo < 300ll * rows_num_sms()) return false;
-        for (int nset = 4; nset >= 2; --nset) tr[n++] = {64, 1, nset};
+        for (int nset = 4; nset >= 2; --nset) tr[n++] = {1, nset};
     } else {
         if (g.C != 64 || (long long)ni * g.H * g.W < 20ll * rows_num_sms()) return false;
-        tr[n++] = {64, 2, 2};
-        tr[n++] = {64, 1, 2};
+        tr[n++] = {2, 2};
+        tr[n++] = {1, 2};
     }
     for (int i = 0; i < n; ++i)
-        if (rows_plan(fwd, g, ni, C_out, Mp, cb_inner, tr[i].BN, tr[i].NT, tr[i].nset, p)) {
+        if (rows_plan(fwd, g, ni, C_out, Mp, cb_inner, tr[i].NT, tr[i].nset, p)) {
             t = tr[i];
             return true;
         }
@@ -1506,7 +1467,6 @@ cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const Lif
     RowsArgs a{};
     a.rec = rec;
     a.C_t = C_t;
-    a.C_out = C_out;
     a.t_out = t_out;
     a.q_out = q;
     a.s_out = s;
@@ -1515,8 +1475,13 @@ cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const Lif
     a.penalty = penalty;
     a.c = c;
     CUtensorMap mB;
-    if (!rows_map_mat(&mB, Wf, C_out, g.k * g.k * g.C, t.BN)) return cudaErrorInvalidValue;
-    return rows_launch<64, 1, true>(mB, mB, a, p, st);
+    if (!rows_map_mat(&mB, Wf, C_out, g.k * g.k * g.C, ROWS_BN)) return cudaErrorInvalidValue;
+    // the generator's code is laid out for its slots (2 or 3 for 3x3 filters, 3 or 4 for 5x5): unrolled for more than
+    // it needs, it overran the instruction cache
+    const int slots = (p.npos + 1) / 2;
+    if (slots <= 2) return rows_launch<1, true, 2>(mB, mB, a, p, st);
+    if (slots <= 3) return rows_launch<1, true, 3>(mB, mB, a, p, st);
+    return rows_launch<1, true, GEN_SLOTS>(mB, mB, a, p, st);
 }
 
 bool conv_rows_ds_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner) {
@@ -1535,15 +1500,14 @@ cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifC
     RowsArgs a{};
     a.t_in = t_in;
     a.C_t = C_t;
-    a.C_out = g.C;
     a.g_t_in = g_t_in;
     a.c = c;
     CUtensorMap mA, mB;
     if (!rows_map_act(&mA, dW_hat, ni, g.Ho, g.Wo, c.Mp, C_out, p.npos) ||
-        !rows_map_mat(&mB, Wt, g.C, g.k * g.k * C_out, t.BN))
+        !rows_map_mat(&mB, Wt, g.C, g.k * g.k * C_out, ROWS_BN))
         return cudaErrorInvalidValue;
-    if (t.NT == 2) return rows_launch<64, 2, false>(mA, mB, a, p, st);
-    return rows_launch<64, 1, false>(mA, mB, a, p, st);
+    if (t.NT == 2) return rows_launch<2, false, 1>(mA, mB, a, p, st);
+    return rows_launch<1, false, 1>(mA, mB, a, p, st);
 }
 
 bool conv_dw_cols_records(int C_out) { return C_out == 64; }

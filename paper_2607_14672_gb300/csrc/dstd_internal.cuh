@@ -104,14 +104,13 @@ __device__ __forceinline__ BinW bin_weights(const LifConst &c, float t, bool der
 // so the lanes of a warp solve together instead of once per interval.
 // ---------------------------------------------------------------------------
 struct ScanState {
-    float v, I;
     int q;       // M while silent
     float v0, I0, hi;  // state at T_q and bracket end of the firing interval
     float s, vdot;
 };
 
 __device__ __forceinline__ void scan_reset(ScanState &st, int M) {
-    st.v = 0.f; st.I = 0.f; st.q = M; st.v0 = 0.f; st.I0 = 0.f; st.hi = 0.f; st.s = 0.f; st.vdot = 0.f;
+    st.q = M; st.v0 = 0.f; st.I0 = 0.f; st.hi = 0.f; st.s = 0.f; st.vdot = 0.f;
 }
 
 __device__ __forceinline__ float vhat_at(const LifConst &c, float v0, float I0, float s) {
@@ -157,9 +156,7 @@ __device__ __forceinline__ float interval_root(const LifConst &c, float v0, floa
 
 // Exact firing test of one interval whose cheap bound reached v_th: the
 // bracket end for the root (0 if v^ is already at v_th at T_q, dt if v^(dt)
-// >= v_th, the interior maximum if only that reaches v_th), or -1. Out of
-// line where it runs once per interval (scan_step), inline where it runs
-// once per block of intervals (scan_block).
+// >= v_th, the interior maximum if only that reaches v_th), or -1.
 __device__ __forceinline__ float interval_test(float av, float aI, float lam, int lam_zero, float rI, float dt,
                                                float vth, float v0, float I0, float ve) {
     if (v0 >= vth) return 0.0f;
@@ -179,61 +176,6 @@ __device__ __forceinline__ float interval_test(float av, float aI, float lam, in
     }
     return -1.0f;
 }
-// Consume w^_m for the SUB intervals m0 .. m0+SUB-1 of one neuron at once,
-// with the grid weights in registers (w[off + j] * rs for interval m0 + j).
-// Same result as SUB calls of scan_step, in two phases so that the lanes of
-// a warp stay together: a branch-free pass runs the recurrence and picks the
-// first interval where v^ reaches v_th at an end point, or has an interior
-// maximum that the cheap bound does not exclude; the exact test then runs
-// once, for all lanes at their own candidate. Only an interior maximum that
-// stays below v_th fails it; the pass then restarts after that interval.
-template <int SUB>
-__device__ __forceinline__ void scan_block(const LifConst &c, ScanState &st, const float (&w)[32], int off, float rs,
-                                           int m0) {
-    if (st.q < c.M) return;
-    const int nvalid = c.M - m0;  // intervals of the block below M
-    if (nvalid <= 0) return;
-    const float v_in = st.v, I_in = st.I;
-    int j0 = 0;
-    for (int pass = 0; pass < SUB; ++pass) {
-        float v = v_in, I = I_in;
-        int cand = SUB;
-        float cv0 = 0.f, cI0 = 0.f, cve = 0.f;
-#pragma unroll
-        for (int j = 0; j < SUB; ++j) {
-            const float I0 = I + w[off + j] * rs;
-            const float ve = c.rv * v + c.KD * I0;
-            // v^ reaches v_th at an end of the interval, or may at an
-            // interior maximum (rising at s = 0, falling at s = dt, bound met)
-            const float d0 = -c.av * v + I0;
-            const float dE = -c.av * ve + c.rI * I0;
-            const bool endp = (v >= c.vth) | (ve >= c.vth);
-            const bool peak = (d0 > 0.0f) & (dE < 0.0f) & (fmaxf(v, 0.0f) + fmaxf(I0, 0.0f) * c.Kmax >= c.vth);
-            const bool take = (cand == SUB) & (j >= j0) & (j < nvalid) & (endp | peak);
-            cand = take ? j : cand;
-            cv0 = take ? v : cv0;
-            cI0 = take ? I0 : cI0;
-            cve = take ? ve : cve;
-            v = ve;
-            I = c.rI * I0;
-        }
-        if (pass == 0) {
-            st.v = v;
-            st.I = I;
-        }
-        if (cand == SUB) return;
-        const float hi = interval_test(c.av, c.aI, c.lam, c.lam_zero, c.rI, c.dt, c.vth, cv0, cI0, cve);
-        if (hi >= 0.0f) {
-            st.q = m0 + cand;
-            st.v0 = cv0;
-            st.I0 = cI0;
-            st.hi = hi;
-            return;
-        }
-        j0 = cand + 1;
-    }
-}
-
 // Root of the firing interval and dv^/dt there (once per neuron).
 __device__ __forceinline__ void scan_finish(const LifConst &c, ScanState &st) {
     if (st.q >= c.M) return;

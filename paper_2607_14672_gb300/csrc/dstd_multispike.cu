@@ -23,9 +23,7 @@ inline unsigned ms_blocks(long long n, int threads) { return (unsigned)((n + thr
 
 template <int OP>
 __device__ __forceinline__ void ms_store(void *hi, void *lo, long long o, float v) {
-    if (OP == 0) {
-        static_cast<float *>(hi)[o] = v;
-    } else if (OP == 3) {
+    if (OP == 3) {
         const __half h = __float2half_rn(v);
         static_cast<__half *>(hi)[o] = h;
         static_cast<__half *>(lo)[o] = __float2half_rn(v - __half2float(h));
@@ -39,9 +37,7 @@ __device__ __forceinline__ void ms_store(void *hi, void *lo, long long o, float 
 // two neighbouring elements, o even (rows of operands start on 16-byte boundaries)
 template <int OP>
 __device__ __forceinline__ void ms_store2(void *hi, void *lo, long long o, float v0, float v1) {
-    if (OP == 0) {
-        *reinterpret_cast<float2 *>(static_cast<float *>(hi) + o) = make_float2(v0, v1);
-    } else if (OP == 3) {
+    if (OP == 3) {
         const __half2 h = __floats2half2_rn(v0, v1);
         *reinterpret_cast<__half2 *>(static_cast<__half *>(hi) + o) = h;
         *reinterpret_cast<__half2 *>(static_cast<__half *>(lo) + o) =
@@ -155,7 +151,7 @@ cudaError_t launch_binning_ms(const float *t, int B, int N, int F, const LifCons
         k_binning_ms_rows<OPV><<<dim3((unsigned)((ld + 255) / 256), (unsigned)B), 128, 0, st>>>(t, B, N, F, c, \
                                                                                                 hi, lo, ld);
     switch (op) {
-        case OpKind::F32: DSTD_MS_BIN(0) break;
+        case OpKind::F32: return cudaErrorInvalidValue;
         case OpKind::BF16X3: DSTD_MS_BIN(1) break;
         case OpKind::BF16: DSTD_MS_BIN(2) break;
         default: DSTD_MS_BIN(3) break;
@@ -361,12 +357,10 @@ __global__ void __launch_bounds__(256) k_dwhat_ms(const float *__restrict__ t_ou
 cudaError_t launch_dwhat_ms(const float *t_out, const int *q, const float *I, const float *vd, const float *g_up,
                             int B, int N, int F, const LifConst &c, OpKind op, void *a_hi, void *a_lo, int lda,
                             void *b_hi, void *b_lo, int ldb, cudaStream_t st) {
-    if (F < 1 || F > kMsMaxSpikes) return cudaErrorInvalidValue;
+    if (F < 1 || F > kMsMaxSpikes || op == OpKind::F32) return cudaErrorInvalidValue;
     const size_t smem = sizeof(float) * ((size_t)c.Mp * (MS_DW_NEURONS + 1) + 4 * MS_DW_NEURONS * F + MS_DW_NEURONS);
     const dim3 g((unsigned)((N + MS_DW_NEURONS - 1) / MS_DW_NEURONS), (unsigned)B);
-    if (op == OpKind::F32)
-        k_dwhat_ms<0><<<g, 256, smem, st>>>(t_out, q, I, vd, g_up, B, N, F, c, a_hi, a_lo, lda, b_hi, b_lo, ldb);
-    else if (op == OpKind::BF16X3)
+    if (op == OpKind::BF16X3)
         k_dwhat_ms<1><<<g, 256, smem, st>>>(t_out, q, I, vd, g_up, B, N, F, c, a_hi, a_lo, lda, b_hi, b_lo, ldb);
     else
         k_dwhat_ms<2><<<g, 256, smem, st>>>(t_out, q, I, vd, g_up, B, N, F, c, a_hi, a_lo, lda, b_hi, b_lo, ldb);
