@@ -13,8 +13,8 @@
 // box serves 36 to 72 MMAs. What bounds this kernel then: dS at 64 channels
 // runs at 53 clocks per N = 64 MMA, of which reading the operands from shared
 // memory takes 48 (64 -> 64 at 28 x 28, B = 256, M = 64: 1.35 -> 0.68 ms); the
-// forward is bound by the scan's instructions (the same layer: 2.38 -> 1.66 ms
-// with the binning).
+// forward is bound by the scan's instructions (issue slots 68% busy, the tensor
+// pipe 27%; the same layer: 2.38 -> 1.66 ms with the binning).
 //
 //   forward  the box holds the binned input and is generated on chip from 8
 //            bytes per input spike (two nonzeros of Mp; generator warps erase
@@ -888,7 +888,8 @@ __global__ void __launch_bounds__(FWD ? FWD_MAX_THREADS : DS_MAX_THREADS, 1)
 // the last three are tiles of their own (TMEM holds four accumulators of 128
 // columns). Split over output rows; fp32 atomics into g_W. Warps: 0 TMA, 1-4
 // MMA issue (block b by warp b mod 4), 5-12 epilogue, 13.. generators. Bound by
-// the MMAs' reads of shared memory. Measured, a box per tap before and by columns
+// the MMAs: the tensor pipe is 55% busy with N = 64, whose operand reads cap it
+// at 67%, and 75% with N = 128. Measured, a box per tap before and by columns
 // (B = 256, M = 64): 64 -> 64 at 28 x 28 1.29 -> 0.92 ms
 // (and 0.27 ms of writing S -> 0.07 of records), 128 -> 128 at 14 x 14 0.79 -> 0.61.
 // ---------------------------------------------------------------------------
@@ -1415,38 +1416,75 @@ cudaError_t rows_launch(const CUtensorMap &mA, const CUtensorMap &mB, const Rows
     return cudaGetLastError();
 }
 
+// Expected time of dS by rows under plan p: launch, and per round of items on
+// the SMs a source box (of one channel block), a pair of a source row and a
+// filter row, its taps, an output row and the item. Fitted, as in
+// conv_ds_tap_us, for each way the filters come (resident, a filter row or one
+// filter column at a time) and each order of the products (2 to 8% rms).
+double rows_ds_us(const RowsPlan &p, int NT) {
+    struct Fit {
+        double launch, box, pair, tap, row, item;
+    };
+    static const Fit fits[2][3][2] = {  // [NT - 1][resident, rows, columns][cb_inner]
+        {{{13.3, 0.857, 0.0, 0.070, 0.0, 0.21}, {10.9, 0.349, 0.0, 0.0, 0.0, 0.0}},
+         {{13.0, 0.806, 0.0, 0.123, 0.156, 0.163}, {13.0, 0.806, 0.0, 0.123, 0.156, 0.163}},
+         {{8.7, 1.667, 0.0, 0.313, 0.0, 0.0}, {13.6, 0.0, 0.0, 0.239, 0.0, 0.55}}},
+        {{{12.7, 0.254, 0.236, 0.0, 1.227, 0.12}, {12.1, 0.079, 0.0, 0.424, 0.0, 0.12}},
+         {{13.1, 0.815, 0.0, 0.100, 0.14, 0.0}, {13.1, 0.815, 0.0, 0.100, 0.14, 0.0}},
+         {{14.0, 0.265, 0.0, 0.156, 0.0, 0.09}, {14.0, 0.265, 0.0, 0.156, 0.0, 0.09}}}};
+    const Fit &f = fits[NT - 1][p.res_bytes ? 0 : (p.kwg > 1 || p.k == 1) ? 1 : 2][p.cb_inner ? 1 : 0];
+    long long src = 0, pairs = 0;  // over the strips of an image's columns
+    for (int s = 0; s < p.n_strip; ++s) {
+        const int ya = s * p.R, yb = ya + p.R < p.gh ? ya + p.R : p.gh;
+        for (int r = 0; r < p.sh; ++r) {  // rows ya .. yb - 1 through filter rows of 0 .. k - 1
+            const int lo = ya > r * p.s - p.pad ? ya : r * p.s - p.pad;
+            const int hi = yb - 1 < r * p.s - p.pad + p.k - 1 ? yb - 1 : r * p.s - p.pad + p.k - 1;
+            if (hi < lo) continue;
+            ++src;
+            pairs += hi - lo + 1;
+        }
+    }
+    const double rounds = (double)((p.n_items + rows_num_sms() - 1) / rows_num_sms()), per = rounds / p.n_strip;
+    return f.launch + per * p.ncb * (f.box * src + pairs * (f.pair + f.tap * p.k * (p.s == 1 ? NT : 1))) +
+           per * f.row * p.gh + f.item * rounds;
+}
+
 struct Tile {
     int NT, nset;
 };
 
-// The tile shapes to try, best first, where this kernel is the faster one.
-// Measured against the one-row-at-a-time kernels (whose issue loops run as
-// whole warps too), every layer shape of the 9- and 20-layer networks:
-//   forward  64 output channels of one channel block at stride 1: 1.01 to 1.07
-//            times faster from about 300 output positions per SM on (binning
-//            included), 0.86 to 0.96 below. Not built: two channel blocks
-//            (0.82), stride 2 (0.95 to 1.02), 128 and more output channels
-//            (filters streamed, 0.6 to 0.9); 1x1 0.91;
-//   dS       64 input channels: 1.2 to 2.3 times faster (64 -> 64 at 28 x 28:
-//            1.55; 64 -> 128 at stride 2: 2.0), 0.87 to 1 on a few thousand
-//            positions; 128 input channels: 0.8 to 0.96, wider: 0.5 to 0.9.
+// Where this kernel is the faster one, measured against the one-row-at-a-time
+// kernels over 3 to 32 wide images:
+//   forward  64 output channels of one channel block at stride 1, from about
+//            300 output positions per SM on: with the filters resident or
+//            streamed a filter row at a time, 2x2 to 4x4 filters 1.02 to 1.54
+//            times faster (3x3 at 28 x 28, M = 64: 1.07 to 1.13, binning
+//            included); 5x5 1.1 to 1.3 where the other kernel has no row boxes
+//            (the position tile does not divide the image's width), 0.85 to 1
+//            where it has; streamed a filter column at a time (4x4 and wider at
+//            64 grid steps, 6x6 and wider) 0.5 to 0.87. Fewer positions 0.86 to
+//            0.96. Not built: two channel blocks (0.82), stride 2 (0.95 to
+//            1.02), 128 and more output channels (0.6 to 0.9); 1x1 0.91;
+//   dS       64 input channels, by the expected times: 64 -> 64 at 28 x 28 and 64
+//            -> 128 at stride 2 1.6 and 2.0 times faster; slower where the tile
+//            is twice as wide as the image (M = 32 at 4 wide, 0.4 to 0.8) and
+//            where the filters stream past row boxes (64 -> 128 at 14 x 14, M = 64:
+//            0.84 to 0.92; 64 -> 64, 7x7: 0.6 to 0.8). Over the fitted layers the
+//            choice costs 0.4% against the better of the two; taken always, these
+//            kernels lost up to 2.4 times.
 bool rows_pick(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner, RowsPlan &p, Tile &t) {
-    Tile tr[3];
-    int n = 0;
     if (fwd) {
         if (C_out != 64 || g.C != 64 || g.s != 1 || g.k == 1) return false;
         if ((long long)ni * g.Ho * g.Wo < 300ll * rows_num_sms()) return false;
-        for (int nset = 4; nset >= 2; --nset) tr[n++] = {1, nset};
+        for (t = Tile{1, 4}; t.nset >= 2; --t.nset)
+            if (rows_plan(true, g, ni, C_out, Mp, cb_inner, t.NT, t.nset, p))
+                return p.res_bytes || (p.kwg > 1 && (g.k < 5 || cb_inner));
     } else {
         if (g.C != 64 || (long long)ni * g.H * g.W < 20ll * rows_num_sms()) return false;
-        tr[n++] = {2, 2};
-        tr[n++] = {1, 2};
+        for (t = Tile{2, 2}; t.NT >= 1; --t.NT)
+            if (rows_plan(false, g, ni, C_out, Mp, cb_inner, t.NT, t.nset, p))
+                return rows_ds_us(p, t.NT) < conv_ds_tap_us(g, ni, C_out, Mp);
     }
-    for (int i = 0; i < n; ++i)
-        if (rows_plan(fwd, g, ni, C_out, Mp, cb_inner, tr[i].NT, tr[i].nset, p)) {
-            t = tr[i];
-            return true;
-        }
     return false;
 }
 

@@ -1,29 +1,35 @@
 // Convolutional DSTD layer as implicit GEMMs on sm_103a (bf16 operands,
-// tcgen05), with no im2col operand and no binned array in memory.
+// tcgen05), with no im2col operand. (The kernels that take each source row or
+// column once are in dstd_conv_rows.cu.)
 //
 // Layouts (a chunk of whole images, NHWC positions p = (b*H + y)*W + x):
-//   rec   [P_in][C_in]       8 B   per input spike: grid step k and the bf16
-//                                  pair of its two weights (Eq. DSTD_kernel)
-//   w^    [P_out][C_out][Mp] fp32  the forward contraction (Eq. DSTD), the
-//                                  Mp grid steps of a neuron contiguous
+//   S     [P_in][Mp][C_in]   bf16  the binned input (Eq. DSTD_kernel): two
+//                                  nonzero grid weights per input spike
+//   rec   [P_in][C_in]       8 B   instead of S: grid step k and the bf16
+//                                  pair of the two weights
+//   w^    [P_out][C_out][Mp] fp32  the forward contraction (Eq. DSTD), only
+//                                  where the operand is generated; else in TMEM
 //   dw^   [P_out][Mp][C_out] bf16  dC/dw^ (implicit-function theorem)
 //   Wf    [C_out][k k C_in]  bf16  filters, taps (kh, kw) then channels
 //   Wt    [C_in][k k C_out]  bf16  the same filters transposed
 //
 //   forward  w^[(p, m), o]  = sum_{tap, c} S[(p + tap), m, c] Wf[o, tap, c]:
-//            the binned operand S is generated in shared memory from the
-//            records of the inputs each tap reads (two nonzeros per input)
+//            S read through TMA boxes shifted per tap, the scan in the
+//            epilogue; or generated in shared memory from the records of the
+//            inputs each tap reads (k_conv_fwd_gen), then a scan kernel
 //   dS       dS[(p', m), c] = sum_{tap, o} dw^[(p' - tap) / s, m, o] Wt[c, tap, o]
 //            (the transposed convolution; one TMA box of a 5-D tensor map
 //            (channel, m, x, y, b) per position and tap, coordinates outside
 //            the image or off the stride grid read zeros), consumed in the
 //            epilogue: dC/dt_j = sum_{m in {k, k+1}} dS[(p', m), c] ds_jm/dt_j
 //   dW       dW[o, tap, c]  = sum_{(p, m)} dw^[(p, m), o] S[(p + tap), m, c]
-//            (both operands MN-major, S generated on chip, split-K)
+//            (both operands MN-major, S by TMA or generated on chip, split-K)
 //
-// One thread issues tcgen05.mma (M = 128, N = BN <= 256, K = 16) into TMEM
-// accumulators. Every mbarrier wait is bounded; an expired wait sets this
-// unit's status word, the role stops, and the CTA still frees its TMEM.
+// tcgen05.mma (M = 128, N = BN <= 256, K = 16) into TMEM accumulators, issued by
+// one elected lane of a warp (k_conv_dw_tma: of four) that runs its loop as a
+// whole; the generating kernels issue from one thread. Every mbarrier wait is
+// bounded; an expired wait sets this unit's status word, the role stops, and
+// the CTA still frees its TMEM.
 #include "dstd_internal.cuh"
 #include "dstd_tc_ptx.cuh"
 
@@ -80,9 +86,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 // (packed fp32, and half-precision compares of the row with q that mask the
 // packed bf16). In three loops (before, across and behind the spikes' rows of a
 // thread's neurons) the lanes of a warp, whose spikes lie apart, ran each loop
-// one after another, 2200 instructions per position of 64 channels and bound
-// by them. B = 256, Mp = 64: 64 channels at 28 x 28 0.40 -> 0.36 ms, 128 channels
-// at 14 x 14 0.32 -> 0.26 ms. Direct stores at 64 channels (0.40) and reading the
+// one after another and were bound by those instructions; now 1380 per position
+// of 64 channels, issue slots 48% busy, 0.6 of HBM speed. B = 256, Mp = 64: 64
+// channels at 28 x 28 0.40 -> 0.36 ms, 128 channels at 14 x 14 0.32 -> 0.26 ms. Direct stores at 64 channels (0.40) and reading the
 // next position's inputs ahead (0.38) are slower.
 // ---------------------------------------------------------------------------
 constexpr int DWHAT_NPT = 4;
@@ -412,7 +418,7 @@ __host__ __device__ constexpr int fwd_epi_bytes(bool tight) { return 2 * 2 * 2 *
 // The two issuing warps run their loops as whole warps (see elect_one): by one
 // lane alone an MMA took about 100 clocks to issue. Forward contraction with
 // the scan, before and after: 128 -> 128 at 14 x 14, B = 256, M = 64: 0.90 ->
-// 0.78 ms; 5x5 128 -> 128 at 8 x 8, B = 50, M = 20: 125 -> 89 us.
+// 0.77 ms; 5x5 128 -> 128 at 8 x 8, B = 50, M = 20: 125 -> 89 us.
 // ---------------------------------------------------------------------------
 template <int BN, bool ROWBOX, bool RES, bool FWD>
 __global__ void __launch_bounds__(CONV_THREADS, 1)
@@ -2057,31 +2063,13 @@ bool conv_ds_row_boxes(const ConvGeom &g, int C_out, int Mp) {
     return rowbox;
 }
 
-// dS of ni images with the input-time gradient: dw^ [ni Ho Wo][Mp][C_out],
-// Wt [C_in][k k C_out], t_in [ni H W][C_in] -> g_t_in (zeroed first)
-cudaError_t launch_conv_ds_gemm(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *dW_hat,
-                                const __nv_bfloat16 *Wt, const float *t_in, float *g_t_in, int C_t, cudaStream_t st) {
-    ConvGemmArgs a = base_args(g, ni, c);
-    a.C_out = C_out;
-    a.P_rows = ni * g.H * g.W;
-    const int BN = pick_bn(g.C);
-    const int ppt = 128 / c.Mp;
-    a.n_col = g.C / BN;
-    a.t_in = t_in;
-    a.g_t_in = g_t_in;
-    a.C_t = C_t;
-    cudaError_t e = cudaMemsetAsync(g_t_in, 0, sizeof(float) * (size_t)a.P_rows * C_t, st);
-    if (e != cudaSuccess) return e;
-    bool resident, rowbox;
-    DsPlan pl = ds_tap_plan(g, C_out, c.Mp, resident, rowbox);
-    if (pl.nst < 2) return cudaErrorInvalidConfiguration;
-    // stride classes (one for stride 1); a stride whose s x s classes do not
-    // fit runs every tap in the identity order, off-grid taps reading zeros
+// the stride classes of dS (one for stride 1); a stride whose s x s classes do
+// not fit runs every tap in the identity order, off-grid taps reading zeros
+static void ds_classes(const ConvGeom &g, int ni, DsPlan &pl) {
     const bool classes = g.s * g.s <= DS_MAX_CLS;
     pl.ps = classes ? g.s : 1;
     pl.ts = classes ? g.s : 1;
     pl.ncls = 0;
-    a.n_row = 0;
     for (int py = 0; py < pl.ps; ++py)
         for (int px = 0; px < pl.ps; ++px) {
             DsClass q{};
@@ -2104,6 +2092,55 @@ cudaError_t launch_conv_ds_gemm(const ConvGeom &g, int ni, int C_out, const LifC
             pl.cls[j] = pl.cls[j - 1];
             pl.cls[j - 1] = q;
         }
+}
+
+// Launch, and per round of tiles on the SMs a unit (one filter row of a channel
+// block with row boxes, else one tap; with row boxes and filters that do not
+// stay resident, a part per tap), a box more where a tile's positions are no
+// run, and a tile's epilogue: fitted to dS of 64 input channels (2198 layers,
+// 1x1 to 7x7, strides 1 and 2, 3 to 32 wide; 3 to 8% rms)
+double conv_ds_tap_us(const ConvGeom &g, int ni, int C_out, int Mp) {
+    bool resident, rowbox;
+    DsPlan pl = ds_tap_plan(g, C_out, Mp, resident, rowbox);
+    ds_classes(g, ni, pl);
+    const int ppt = 128 / Mp, ncb = C_out / 64, sms = conv_num_sms();
+    double tiles = 0.0, units = 0.0, boxes = 0.0;
+    for (int i = 0; i < pl.ncls; ++i) {
+        const DsClass &q = pl.cls[i];
+        const double n = (q.count + ppt - 1) / ppt, u = (double)(rowbox ? g.k : q.nkh * q.nkw) * ncb;
+        int broken = 0;
+        for (int j = 0; j < q.Wc; ++j) broken += (int)((long long)j * ppt % q.Wc) + ppt > q.Wc;
+        tiles += n;
+        units += n * u;
+        boxes += rowbox ? 0.0 : n * u * broken / q.Wc * (ppt - 1);
+    }
+    if (tiles == 0.0) return 0.0;
+    const double rounds = (double)(((long long)tiles * (g.C / pick_bn(g.C)) + sms - 1) / sms), f = rounds / tiles;
+    if (!rowbox) return 10.9 + f * (0.208 * units + 0.036 * boxes) + 1.15 * rounds;
+    return resident ? 9.9 + f * 0.221 * units + 1.01 * rounds
+                    : 10.2 + f * (0.153 + 0.104 * g.k) * units + 0.33 * rounds;
+}
+
+// dS of ni images with the input-time gradient: dw^ [ni Ho Wo][Mp][C_out],
+// Wt [C_in][k k C_out], t_in [ni H W][C_in] -> g_t_in (zeroed first)
+cudaError_t launch_conv_ds_gemm(const ConvGeom &g, int ni, int C_out, const LifConst &c, const __nv_bfloat16 *dW_hat,
+                                const __nv_bfloat16 *Wt, const float *t_in, float *g_t_in, int C_t, cudaStream_t st) {
+    ConvGemmArgs a = base_args(g, ni, c);
+    a.C_out = C_out;
+    a.P_rows = ni * g.H * g.W;
+    const int BN = pick_bn(g.C);
+    const int ppt = 128 / c.Mp;
+    a.n_col = g.C / BN;
+    a.t_in = t_in;
+    a.g_t_in = g_t_in;
+    a.C_t = C_t;
+    cudaError_t e = cudaMemsetAsync(g_t_in, 0, sizeof(float) * (size_t)a.P_rows * C_t, st);
+    if (e != cudaSuccess) return e;
+    bool resident, rowbox;
+    DsPlan pl = ds_tap_plan(g, C_out, c.Mp, resident, rowbox);
+    if (pl.nst < 2) return cudaErrorInvalidConfiguration;
+    ds_classes(g, ni, pl);
+    a.n_row = 0;
     for (int i = 0; i < pl.ncls; ++i) {
         pl.cls[i].tile0 = a.n_row;
         a.n_row += (pl.cls[i].count + ppt - 1) / ppt;

@@ -514,6 +514,8 @@ cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const Lif
 bool conv_rows_ds_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner);
 cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
                                 const __nv_bfloat16 *dW_hat, const __nv_bfloat16 *Wt, const float *t_in, float *g_t_in, int C_t, cudaStream_t st);
+// expected time of launch_conv_ds_gemm
+double conv_ds_tap_us(const ConvGeom &g, int ni, int C_out, int Mp);
 // dW of 3x3 layers at stride 1, each column of S taken once per channel block
 // (same file; as launch_conv_dw_tma): generated from the records [ni H W][C_t]
 // where conv_dw_cols_records says so, else (rec null) read from S. pick:

@@ -1,9 +1,10 @@
 """Which kernels a conv layer takes (dstd_conv_route): the rules on the host, and, on the GPU, that the shapes meant
 to check the kernels by source rows against the one-row-at-a-time kernels do take them.
 
-Forward by rows: 64 output channels, one block of 64 input channels (or fewer, padded), stride 1, filters above 1x1,
-300 output positions per SM. dS by rows: one block of input channels, 20 input positions per SM, at most eight output
-rows in flight (four at stride 2). Forward results are equal bit for bit, input-time gradients to 1e-5 relative L2
+Forward by rows: 64 output channels, one block of 64 input channels (or fewer, padded), stride 1, filters above 1x1
+that come at least a filter row at a time, 300 output positions per SM. dS by rows: one block of input channels, 20
+input positions per SM, at most eight output rows in flight (four at stride 2). Both only where they are the faster
+kernels, as the measured times say. Forward results are equal bit for bit, input-time gradients to 1e-5 relative L2
 (the two bins of an input may be added in either order), as in test_gpu_conv_rows.py.
 
 dW by columns: 3x3 at stride 1, 64 output channels, or a multiple of 128 with 64 grid steps, on the side of the
@@ -25,15 +26,26 @@ LARGE = [
     (1, 6, 64, 64, 3, 1, 1, 32, (INF, INF), {"fwd_rows", "ds_rows"}),
     (6, 6, 3, 64, 3, 1, 1, 32, (INF, INF), {"fwd_rows", "ds_rows"}),
     (8, 8, 64, 64, 2, 1, 1, 32, (INF, INF), {"fwd_rows", "ds_rows"}),
-    (8, 8, 64, 64, 5, 1, 2, 20, (INF, INF), {"fwd_rows", "ds_rows"}),
-    (9, 9, 64, 64, 7, 1, 3, 32, (0.5, 0.25), {"fwd_rows", "ds_rows"}),
+    (9, 9, 64, 64, 4, 1, 2, 32, (INF, INF), {"fwd_rows", "ds_rows"}),     # filters a row at a time
+    (7, 7, 64, 64, 5, 1, 2, 20, (INF, INF), {"fwd_rows", "ds_rows"}),
+    (4, 4, 64, 64, 3, 1, 1, 32, (0.5, 0.25), {"fwd_rows"}),              # dS tiles twice as wide as the image
+    (9, 9, 64, 64, 7, 1, 3, 32, (0.5, 0.25), {"ds_rows"}),               # filters a column at a time: no forward
+    (7, 7, 64, 64, 5, 1, 2, 64, (0.5, 0.25), {"ds_rows"}),
     (8, 8, 64, 64, 1, 1, 0, 32, (INF, INF), {"ds_rows"}),
     (9, 9, 64, 128, 3, 2, 1, 64, (1.0, 0.25), {"ds_rows"}),
     (10, 10, 64, 64, 3, 2, 1, 32, (INF, INF), {"ds_rows"}),
     (7, 9, 64, 128, 3, 1, 1, 64, (0.5, 0.25), {"ds_rows"}),
+    (7, 7, 64, 128, 3, 1, 1, 32, (0.5, 0.25), {"ds_rows"}),
+    (4, 4, 64, 128, 3, 1, 1, 64, (0.5, 0.25), {"ds_rows"}),
     (8, 8, 64, 256, 3, 1, 1, 32, (0.5, 0.25), {"ds_rows"}),
-    (7, 7, 64, 256, 3, 1, 1, 32, (0.5, 0.25), set()),    # four channel blocks in one stage: too large
+    (3, 3, 64, 256, 1, 1, 0, 32, (0.5, 0.25), {"ds_rows"}),
+    (4, 4, 64, 512, 5, 1, 2, 64, (0.5, 0.25), {"ds_rows"}),
+    (7, 7, 64, 256, 3, 1, 1, 32, (0.5, 0.25), set()),                    # four channel blocks in one stage: too large
     (9, 9, 64, 64, 5, 2, 2, 64, (0.5, 0.25), set()),     # six output rows in flight, four accumulators
+    (28, 28, 64, 128, 3, 1, 1, 32, (1.0, 0.25), set()),  # from here on: 0.6 to 0.9 of the other kernels' speed
+    (28, 28, 64, 64, 5, 1, 2, 20, (INF, INF), set()),    # (those have row boxes)
+    (28, 28, 64, 64, 5, 1, 2, 64, (1.0, 0.25), set()),
+    (28, 28, 64, 64, 7, 1, 3, 64, (1.0, 0.25), set()),
     (14, 14, 128, 128, 3, 1, 1, 64, (1.0, 0.25), set()),
     (14, 14, 128, 64, 3, 1, 1, 64, (1.0, 0.25), set()),
 ]
@@ -143,7 +155,7 @@ def test_rows_are_taken_and_match(lib, case):
     dstd.device_status(clear=True)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     Ho, Wo = dstd.conv_out_hw(case[0], case[1], *case[4:7])
-    B = (300 * sms // (Ho * Wo) if "fwd_rows" in case[9] else 20 * sms // (case[0] * case[1])) + 1
+    B = (300 * sms // (Ho * Wo) if "fwd_rows" in case[9] else 60 * sms // (case[0] * case[1])) + 1
     assert route(B, case) & ROWS == case[9] and route(B, case, policy=2) & ROWS == set()
     a, b = run(B, *case[:9], policy=0), run(B, *case[:9], policy=2)
     assert torch.isfinite(a[0]).any() and (a[3] != 0).any()
