@@ -719,10 +719,11 @@ struct ConvFwdRoute {
     bool rows;      // by source rows, from records (in S's place, which is larger)
     bool cb_inner;  // order of its products (see conv_fwd_row_boxes)
 };
-static ConvFwdRoute conv_fwd_route(const ConvGeom &g, int ni, int C_out, int Mp) {
+static ConvFwdRoute conv_fwd_route(const ConvGeom &g, int ni, int C_out, int Mp, const dstd_params &p) {
     const ConvGeom gp = conv_padded(g);
+    const float decay = (p.t_end - p.t_first) / fmaxf(p.tau_m, p.tau_s);
     ConvFwdRoute r{conv_fwd_tma(g, C_out), false, !conv_fwd_row_boxes(gp, C_out, Mp)};
-    r.rows = r.S && g_conv_operand_policy == 0 && conv_rows_fwd_supported(gp, ni, C_out, Mp, r.cb_inner);
+    r.rows = r.S && g_conv_operand_policy == 0 && conv_rows_fwd_faster(gp, ni, C_out, Mp, r.cb_inner, decay);
     if (r.rows) r.S = false;
     return r;
 }
@@ -736,7 +737,7 @@ static ConvBwdRoute conv_bwd_route(const ConvGeom &g, int ni, int C_out, int Mp)
     const ConvGeom gp = conv_padded(g);
     ConvBwdRoute r{false, !conv_ds_row_boxes(gp, C_out, Mp), false, conv_dw_tma(g, C_out), {}};
     if (g_conv_operand_policy != 0) return r;
-    r.ds_rows = conv_rows_ds_supported(gp, ni, C_out, Mp, r.ds_cb_inner);
+    r.ds_rows = conv_rows_ds_faster(gp, ni, C_out, Mp, r.ds_cb_inner);
     r.dw_cols = r.dw_S && conv_dw_cols_pick(gp, ni, C_out, Mp, g.C, r.dw_split);
     if (r.dw_cols && conv_dw_cols_records(C_out)) r.dw_S = false;
     return r;
@@ -767,7 +768,7 @@ int conv_fwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
     }
     for (int img0 = 0; img0 < g.B; img0 += ws.imgs) {
         const int ni = (g.B - img0) < ws.imgs ? (g.B - img0) : ws.imgs;
-        const ConvFwdRoute rt = conv_fwd_route(g, ni, C_out, Mp);
+        const ConvFwdRoute rt = conv_fwd_route(g, ni, C_out, Mp, *p);
         const long long in_off = (long long)img0 * g.H * g.W * g.C;
         const long long out_off = (long long)img0 * g.Ho * g.Wo * C_out;
         const long long P_out = (long long)ni * g.Ho * g.Wo;
@@ -1231,7 +1232,7 @@ int dstd_conv_route(int B, int H, int W, int C_in, int C_out, int k, int stride,
     TRY(conv_plan(B, H, W, C_in, k, stride, pad, Mp, true, C_out, &pl));
     if (!conv_use_implicit(math, pl.g, C_out, Mp)) return 0;
     const int ni = conv_impl_images(pl.g, C_out, Mp);
-    const ConvFwdRoute f = conv_fwd_route(pl.g, ni, C_out, Mp);
+    const ConvFwdRoute f = conv_fwd_route(pl.g, ni, C_out, Mp, *p);
     const ConvBwdRoute b = conv_bwd_route(pl.g, ni, C_out, Mp);
     return DSTD_ROUTE_IMPLICIT | (f.S || f.rows ? DSTD_ROUTE_FUSED_SCAN : 0) | (f.rows ? DSTD_ROUTE_FWD_ROWS : 0) |
            (f.S ? DSTD_ROUTE_FWD_BINNED : 0) | (b.ds_rows ? DSTD_ROUTE_DS_ROWS : 0) |

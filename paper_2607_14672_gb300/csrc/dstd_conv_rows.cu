@@ -1463,8 +1463,12 @@ struct Tile {
 //            (the position tile does not divide the image's width), 0.85 to 1
 //            where it has; streamed a filter column at a time (4x4 and wider at
 //            64 grid steps, 6x6 and wider) 0.5 to 0.87. Fewer positions 0.86 to
-//            0.96. Not built: two channel blocks (0.82), stride 2 (0.95 to
-//            1.02), 128 and more output channels (0.6 to 0.9); 1x1 0.91;
+//            0.96. With 64 grid steps and little decay over the window (the
+//            lesser rate times its length below 0.9) the scan is light and this
+//            kernel only pays for 3x3 and wider where the other has no row boxes
+//            (1.1 to 1.3; else 0.84 to 1.05). Not built: two channel blocks
+//            (0.82), stride 2 (0.95 to 1.02), 128 and more output channels (0.6
+//            to 0.9); 1x1 0.91;
 //   dS       64 input channels, by the expected times: 64 -> 64 at 28 x 28 and 64
 //            -> 128 at stride 2 1.6 and 2.0 times faster; slower where the tile
 //            is twice as wide as the image (M = 32 at 4 wide, 0.4 to 0.8) and
@@ -1472,28 +1476,35 @@ struct Tile {
 //            0.84 to 0.92; 64 -> 64, 7x7: 0.6 to 0.8). Over the fitted layers the
 //            choice costs 0.4% against the better of the two; taken always, these
 //            kernels lost up to 2.4 times.
+bool rows_faster(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner, float decay,
+                 const RowsPlan &p, const Tile &t) {
+    if (!fwd) return rows_ds_us(p, t.NT) < conv_ds_tap_us(g, ni, C_out, Mp);
+    if (!p.res_bytes && !(p.kwg > 1 && (g.k < 5 || cb_inner))) return false;
+    return Mp < 64 || decay >= 0.9f || (g.k > 2 && cb_inner);
+}
+
+// the plan of a shape that the kernel takes: the most epilogue warps, or the
+// widest tile, that fits
 bool rows_pick(bool fwd, const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner, RowsPlan &p, Tile &t) {
     if (fwd) {
         if (C_out != 64 || g.C != 64 || g.s != 1 || g.k == 1) return false;
         if ((long long)ni * g.Ho * g.Wo < 300ll * rows_num_sms()) return false;
         for (t = Tile{1, 4}; t.nset >= 2; --t.nset)
-            if (rows_plan(true, g, ni, C_out, Mp, cb_inner, t.NT, t.nset, p))
-                return p.res_bytes || (p.kwg > 1 && (g.k < 5 || cb_inner));
+            if (rows_plan(true, g, ni, C_out, Mp, cb_inner, t.NT, t.nset, p)) return true;
     } else {
         if (g.C != 64 || (long long)ni * g.H * g.W < 20ll * rows_num_sms()) return false;
         for (t = Tile{2, 2}; t.NT >= 1; --t.NT)
-            if (rows_plan(false, g, ni, C_out, Mp, cb_inner, t.NT, t.nset, p))
-                return rows_ds_us(p, t.NT) < conv_ds_tap_us(g, ni, C_out, Mp);
+            if (rows_plan(false, g, ni, C_out, Mp, cb_inner, t.NT, t.nset, p)) return true;
     }
     return false;
 }
 
 }  // namespace
 
-bool conv_rows_fwd_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner) {
+bool conv_rows_fwd_faster(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner, float decay) {
     RowsPlan p;
     Tile t;
-    return rows_pick(true, g, ni, C_out, Mp, cb_inner, p, t);
+    return rows_pick(true, g, ni, C_out, Mp, cb_inner, p, t) && rows_faster(true, g, ni, C_out, Mp, cb_inner, decay, p, t);
 }
 
 cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
@@ -1522,10 +1533,10 @@ cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const Lif
     return rows_launch<1, true, GEN_SLOTS>(mB, mB, a, p, st);
 }
 
-bool conv_rows_ds_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner) {
+bool conv_rows_ds_faster(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner) {
     RowsPlan p;
     Tile t;
-    return rows_pick(false, g, ni, C_out, Mp, cb_inner, p, t);
+    return rows_pick(false, g, ni, C_out, Mp, cb_inner, p, t) && rows_faster(false, g, ni, C_out, Mp, cb_inner, 0.f, p, t);
 }
 
 cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,

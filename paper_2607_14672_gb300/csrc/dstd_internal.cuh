@@ -506,12 +506,13 @@ bool conv_ds_row_boxes(const ConvGeom &g, int C_out, int Mp);  // the same of dS
 // The forward and dS contractions that take each source row once
 // (dstd_conv_rows.cu): same results (the forward generates the binned input on
 // chip from the records of launch_bin_rec, [ni H W][C_t]; cb_inner as conv_fwd_row_boxes says, so that
-// w^ is the same bit for bit). supported: the shapes they take.
-bool conv_rows_fwd_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner);
+// w^ is the same bit for bit). faster: the shapes they are taken for. decay:
+// the lesser of the two rates times the window's length
+bool conv_rows_fwd_faster(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner, float decay);
 cudaError_t launch_conv_rows_fwd(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
                                  const uint2 *rec, int C_t, const __nv_bfloat16 *Wf, const float *rowsum,
                                  float *t_out, int *q, float *s, float *vdot, float *penalty, cudaStream_t st);
-bool conv_rows_ds_supported(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner);
+bool conv_rows_ds_faster(const ConvGeom &g, int ni, int C_out, int Mp, bool cb_inner);
 cudaError_t launch_conv_rows_ds(const ConvGeom &g, int ni, int C_out, const LifConst &c, bool cb_inner,
                                 const __nv_bfloat16 *dW_hat, const __nv_bfloat16 *Wt, const float *t_in, float *g_t_in, int C_t, cudaStream_t st);
 // expected time of launch_conv_ds_gemm

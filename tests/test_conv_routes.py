@@ -28,6 +28,9 @@ LARGE = [
     (8, 8, 64, 64, 2, 1, 1, 32, (INF, INF), {"fwd_rows", "ds_rows"}),
     (9, 9, 64, 64, 4, 1, 2, 32, (INF, INF), {"fwd_rows", "ds_rows"}),     # filters a row at a time
     (7, 7, 64, 64, 5, 1, 2, 20, (INF, INF), {"fwd_rows", "ds_rows"}),
+    (7, 7, 64, 64, 3, 1, 1, 64, (INF, INF), {"fwd_rows", "ds_rows"}),
+    (28, 28, 64, 64, 3, 1, 1, 32, (INF, INF), {"fwd_rows", "ds_rows"}),
+    (28, 28, 64, 64, 3, 1, 1, 64, (INF, INF), {"ds_rows"}),              # a light scan beside row boxes
     (4, 4, 64, 64, 3, 1, 1, 32, (0.5, 0.25), {"fwd_rows"}),              # dS tiles twice as wide as the image
     (9, 9, 64, 64, 7, 1, 3, 32, (0.5, 0.25), {"ds_rows"}),               # filters a column at a time: no forward
     (7, 7, 64, 64, 5, 1, 2, 64, (0.5, 0.25), {"ds_rows"}),
