@@ -367,10 +367,10 @@ int dstd_conv_set_chunk_images(int max_images);
  * faster, kernels that take each source row or column once (the forward of
  * large 64 -> 64 layers at stride 1, dS with 64 input channels, dW of 3x3
  * layers at stride 1 with 64 output channels, or a multiple of 128 and
- * 32 < M <= 64), else S wherever its writer takes the channel count
- * (C_in <= 256, or a multiple of 256 up to 1024) and generated elsewhere. All
- * compute the same products. It changes the workspace size, so query again
- * after setting it. Returns the previous value (a policy outside 0..2 only reads it).
+ * 32 < M <= 64; dstd_conv_route says which a layer gets), else S wherever its
+ * writer takes the channel count (C_in <= 256, or a multiple of 256 up to 1024)
+ * and generated elsewhere. All compute the same products. It changes the
+ * workspace size, so query again after setting it. Returns the previous value (a policy outside 0..2 only reads it).
  * Process-wide; set it between calls. */
 int dstd_conv_set_operand_policy(int policy);
 

@@ -1027,10 +1027,14 @@ static cudaError_t launch_pair(const CUtensorMap &a_hi, const CUtensorMap &a_lo,
 // of 128 x 128 tiles on single CTAs, (K steps + 2) each, against rounds of
 // 256 x 128 tiles on resident SM pairs, (0.92 K steps + 4) each. A pair's K
 // step is cheaper (each SM takes in 48 KB instead of 64 KB of operands), its
-// tile boundary dearer (the handshakes between the two SMs); fitted to the
+// tile boundary dearer (the handshakes between the two SMs); fitted in x3 to the
 // 784-wide forward of the MLP (13 K steps: single CTAs faster) and 4096- and
-// 8192-wide layers (64 and 128 K steps: pairs faster, 85-90% against 83% of
-// the bf16 peak).
+// 8192-wide layers (64 and 128 K steps: pairs faster). In bf16 a pair's K step
+// costs less than the model says, since four warps issue it: pairs are taken
+// where they are the slower ones only in small products (dS of 512 inputs x 4096
+// columns, K = 4096: 30 us against 27), but they would also win at 13 to 32 K steps
+// of many tiles (dS of 8192 inputs x 8192 columns, K = 1600: 263 us on single
+// CTAs, 230 on pairs; dW of 8192 x 8192, K = 1024: 194 and 140).
 static std::atomic<int> g_pair_policy{0};
 
 int tc_gemm_pair_policy(int policy) {
