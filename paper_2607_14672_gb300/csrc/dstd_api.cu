@@ -733,12 +733,13 @@ struct ConvBwdRoute {
     bool dw_S;                  // dW reads the binned input written out, else records
     ConvDwColsSplit dw_split;   // of dW by columns
 };
-static ConvBwdRoute conv_bwd_route(const ConvGeom &g, int ni, int C_out, int Mp) {
+static ConvBwdRoute conv_bwd_route(const ConvGeom &g, int ni, int C_out, int Mp, const dstd_params &p) {
     const ConvGeom gp = conv_padded(g);
     ConvBwdRoute r{false, !conv_ds_row_boxes(gp, C_out, Mp), false, conv_dw_tma(g, C_out), {}};
     if (g_conv_operand_policy != 0) return r;
+    const bool decay = isfinite(p.tau_m) || isfinite(p.tau_s);
     r.ds_rows = conv_rows_ds_faster(gp, ni, C_out, Mp, r.ds_cb_inner);
-    r.dw_cols = r.dw_S && conv_dw_cols_pick(gp, ni, C_out, Mp, g.C, r.dw_split);
+    r.dw_cols = r.dw_S && conv_dw_cols_pick(gp, ni, C_out, Mp, g.C, decay, r.dw_split);
     if (r.dw_cols && conv_dw_cols_records(C_out)) r.dw_S = false;
     return r;
 }
@@ -829,7 +830,7 @@ int conv_bwd_implicit(const float *t_in, const float *W, const ConvGeom &g, int 
     for (int img0 = 0; img0 < g.B; img0 += ws.imgs) {
         const int ni = (g.B - img0) < ws.imgs ? (g.B - img0) : ws.imgs;
         const bool last = img0 + ni >= g.B;
-        const ConvBwdRoute rt = conv_bwd_route(g, ni, C_out, Mp);
+        const ConvBwdRoute rt = conv_bwd_route(g, ni, C_out, Mp, *p);
         const long long in_off = (long long)img0 * g.H * g.W * g.C;
         const long long out_off = (long long)img0 * g.Ho * g.Wo * C_out;
         const long long P_out = (long long)ni * g.Ho * g.Wo;
@@ -1233,7 +1234,7 @@ int dstd_conv_route(int B, int H, int W, int C_in, int C_out, int k, int stride,
     if (!conv_use_implicit(math, pl.g, C_out, Mp)) return 0;
     const int ni = conv_impl_images(pl.g, C_out, Mp);
     const ConvFwdRoute f = conv_fwd_route(pl.g, ni, C_out, Mp, *p);
-    const ConvBwdRoute b = conv_bwd_route(pl.g, ni, C_out, Mp);
+    const ConvBwdRoute b = conv_bwd_route(pl.g, ni, C_out, Mp, *p);
     return DSTD_ROUTE_IMPLICIT | (f.S || f.rows ? DSTD_ROUTE_FUSED_SCAN : 0) | (f.rows ? DSTD_ROUTE_FWD_ROWS : 0) |
            (f.S ? DSTD_ROUTE_FWD_BINNED : 0) | (b.ds_rows ? DSTD_ROUTE_DS_ROWS : 0) |
            (b.dw_cols ? DSTD_ROUTE_DW_COLUMNS : 0) | (b.dw_S ? DSTD_ROUTE_DW_BINNED : 0);

@@ -1597,33 +1597,35 @@ static ConvDwColsSplit dw_cols_split(const ConvGeom &g, int ni, int C_out) {
 // it. Measured, a box per tap / by columns (with 64 output channels S or the
 // records included), us: 64 -> 64, M = 64: 12 images of 2 x 2 25 / 23, 250 of
 // 2 x 2 26 / 35, one of 28 x 28 26 / 39, 20 of 14 x 14 46 / 47, 82 of 14 x 14
-// 150 / 108, 82 of 28 x 28 520 / 349; 128 -> 64, M = 32: 40 of 10 x 10 49 / 63;
-// 128 -> 128: 12 of 2 x 2 23 / 16, 250 of 2 x 2 35 / 51, 20 of 14 x 14 64 / 82, 163 of
-// 14 x 14 480 / 414; 256 -> 256: 50 of 2 x 2 27 / 46, 82 of 14 x 14 841 / 756; 512 ->
-// 512: 62 of 4 x 4 213 / 241. The times are fitted as in conv_dw_tma_us (3% rms):
-// launch, a position of a row, a row's two more columns, a tile's epilogue; S
-// at 5.7 TB/s, the records at 2.5.
-// Over the fitted shapes the choice costs 0.3% against the better of the two.
-bool conv_dw_cols_pick(const ConvGeom &g, int ni, int C_out, int Mp, int C_t, ConvDwColsSplit &sp) {
+// 150 / 108, 82 of 28 x 28 520 / 349; M = 32: 165 of 11 x 11 116 / 107;
+// 128 -> 64, M = 32: 40 of 10 x 10 49 / 63; 128 -> 128: 12 of 2 x 2 23 / 16, 250 of
+// 2 x 2 35 / 51, 20 of 14 x 14 64 / 82, 163 of 14 x 14 480 / 414; 256 -> 256: 50 of
+// 2 x 2 27 / 46, 82 of 14 x 14 841 / 756; 512 -> 512: 62 of 4 x 4 213 / 241. The
+// times are fitted as in conv_dw_tma_us (3% rms): launch, a position of a row, a
+// row's two more columns, a tile's epilogue; S at 5.7 TB/s, the records at 2.5, or
+// 4.3 with no decay at all (no exponentials).
+// Over the fitted shapes the choice costs 0.2% against the better of the two.
+// Where both are expected within 2% it stays by columns.
+bool conv_dw_cols_pick(const ConvGeom &g, int ni, int C_out, int Mp, int C_t, bool decay, ConvDwColsSplit &sp) {
     if (g.k != 3 || g.s != 1 || g.C % 64 != 0) return false;
     if (!(C_out == 64 && (Mp == 32 || Mp == 64)) && !(C_out % 128 == 0 && Mp == 64)) return false;
     sp = dw_cols_split(g, ni, C_out);
     struct Fit {
         double launch, pos, row, epi;
     };
-    const Fit f = C_out != 64 ? Fit{8.2, 0.403, 0.292, 6.40}
-                  : Mp == 64  ? Fit{9.2, 0.611, 0.513, 6.34}
-                  : C_t < 64  ? Fit{8.6, 0.489, 0.550, 6.16}   // (its generators have less to write)
-                              : Fit{8.8, 0.537, 0.631, 5.58};
+    const Fit f = C_out != 64 ? Fit{8.2, 0.406, 0.285, 6.42}
+                  : Mp == 64  ? Fit{9.0, 0.623, 0.473, 6.42}
+                  : C_t < 64  ? Fit{8.5, 0.486, 0.560, 6.19}   // (its generators have less to write)
+                              : Fit{9.0, 0.538, 0.641, 5.33};
     const double rounds = (double)((sp.n_tiles + rows_num_sms() - 1) / rows_num_sms());
     double cols = f.launch + rounds * (sp.rows_per * (g.Wo * f.pos + f.row) + f.epi);
     double taps = conv_dw_tma_us(g, ni, C_out, Mp);
     if (conv_dw_cols_records(C_out)) {
         const double in_mb = 1e-6 * ni * g.H * g.W;
-        cols += 5.5 + in_mb * C_t * 12 * 0.405;
+        cols += 5.5 + in_mb * C_t * 12 * (decay ? 0.405 : 0.233);
         taps += 6.3 + in_mb * g.C * Mp * 2 * 0.177;
     }
-    return cols < taps;
+    return 0.98 * cols < taps;
 }
 
 cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const ConvDwColsSplit &sp,

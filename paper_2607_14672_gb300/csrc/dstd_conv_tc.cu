@@ -2272,24 +2272,27 @@ static void dw_tma_tiles(const ConvGeom &g, int C_out, int Mp, ConvGemmArgs &a) 
     a.n_split = (a.ktiles + a.kt_per_split - 1) / a.kt_per_split;
 }
 
-// Launch, and per round of tiles on the SMs a K step (a part of its own, and
-// one per row tile of the CTA) and a row tile's epilogue: fitted to 3x3 layers
-// at stride 1 of 24 to 128000 positions, 64 to 512 channels (2307 times, 5% rms)
+// Launch; per round of tiles on the SMs a K step (a part of its own, and one per
+// row tile of the CTA) and a row tile's epilogue; per tile over the SMs a K step's
+// row tile (a last round of few tiles runs faster, the chip's bandwidth being
+// theirs) less what the start of a tile hides: fitted to 3x3 layers at stride 1
+// of 24 to 128000 positions, 64 to 512 channels (3891 times, 4 to 5% rms)
 double conv_dw_tma_us(const ConvGeom &g, int ni, int C_out, int Mp) {
     ConvGemmArgs a{};
     a.P_rows = ni * g.Ho * g.Wo;
     dw_tma_tiles(g, C_out, Mp, a);
     struct Fit {
-        double launch, step, step_row, epi_row;
+        double launch, step, step_row, epi_row, share_step, share;
     };
     const int BN = pick_bn(C_out);
-    const Fit f = BN == 256   ? Fit{14.6, 0.113, 0.225, 2.03}
-                  : BN == 128 ? Fit{9.7, 0.052, 0.156, 1.54}
-                  : Mp == 64  ? Fit{10.5, 0.356, 0.040, 0.22}
-                              : Fit{9.8, 0.391, 0.053, 0.92};
+    const Fit f = BN == 256   ? Fit{15.9, 0.075, 0.150, 2.19, 0.143, 0.95}
+                  : BN == 128 ? Fit{10.6, 0.030, 0.090, 2.24, 0.091, 1.11}
+                  : Mp == 64  ? Fit{11.6, 0.243, 0.023, 0.51, 0.066, 0.64}
+                              : Fit{11.4, 0.282, 0.021, 1.23, 0.085, 0.93};
     const long long tiles = (long long)a.n_row * a.n_col * a.n_split;
     const double rounds = (double)((tiles + conv_num_sms() - 1) / conv_num_sms());
-    return f.launch + rounds * (a.kt_per_split * (f.step + f.step_row * a.groups) + f.epi_row * a.groups);
+    return f.launch + rounds * (a.kt_per_split * (f.step + f.step_row * a.groups) + f.epi_row * a.groups) +
+           (double)tiles / conv_num_sms() * a.groups * (f.share_step * a.kt_per_split - f.share);
 }
 
 // dW of ni images from the binned input S [ni H W][Mp][C_in] and dw^

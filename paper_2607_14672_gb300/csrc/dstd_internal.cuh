@@ -520,11 +520,12 @@ double conv_ds_tap_us(const ConvGeom &g, int ni, int C_out, int Mp);
 // dW of 3x3 layers at stride 1, each column of S taken once per channel block
 // (same file; as launch_conv_dw_tma): generated from the records [ni H W][C_t]
 // where conv_dw_cols_records says so, else (rec null) read from S. pick:
-// whether it is the faster one, and how its rows are split
+// whether it is the faster one, and how its rows are split (decay: a finite
+// time constant)
 struct ConvDwColsSplit {
     int rows_per, n_tiles;  // output rows of a range, and ranges x tiles of one
 };
-bool conv_dw_cols_pick(const ConvGeom &g, int ni, int C_out, int Mp, int C_t, ConvDwColsSplit &sp);
+bool conv_dw_cols_pick(const ConvGeom &g, int ni, int C_out, int Mp, int C_t, bool decay, ConvDwColsSplit &sp);
 bool conv_dw_cols_records(int C_out);
 cudaError_t launch_conv_dw_cols(const ConvGeom &g, int ni, int C_out, const LifConst &c, const ConvDwColsSplit &sp,
                                 const uint2 *rec, const __nv_bfloat16 *S, const __nv_bfloat16 *dW_hat,

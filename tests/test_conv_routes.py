@@ -61,6 +61,7 @@ COLUMNS = [
     (12, 2, 2, 64, 64, 1, 32), (25, 1, 1, 64, 64, 1, 32), (12, 2, 2, 64, 64, 1, 64),
     (3, 4, 3, 192, 64, 1, 20), (2, 6, 5, 5, 64, 0, 32), (12, 2, 2, 128, 128, 1, 64), (25, 1, 1, 128, 128, 1, 64),
     (2, 3, 4, 64, 128, 1, 50), (3, 2, 2, 128, 256, 2, 33), (800, 5, 4, 64, 64, 2, 40), (700, 9, 9, 64, 128, 0, 64),
+    (347, 11, 11, 64, 64, 1, 32), (195, 16, 16, 64, 64, 1, 32), (92, 24, 24, 64, 64, 1, 32),
 ]
 # ... and clearly slower
 TAPS = [
